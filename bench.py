@@ -97,7 +97,7 @@ class Clocks:
         os.close(fd)
         try:
             self.proc = subprocess.Popen(["nvidia-smi", f"--query-gpu={self.FIELDS}", "--format=csv,noheader,nounits",
-                                          "-i", str(self.idx), "-lms", "200"], stdout=open(self.path, "w"),
+                                          "-i", str(self.idx), "-lms", "20"], stdout=open(self.path, "w"),
                                          stderr=subprocess.DEVNULL)
         except OSError:
             self.proc = None
@@ -178,12 +178,11 @@ def shell32_config(symmetry: int = 0, world: int = 1) -> dict:
     """`config` of the headline line, shared by both arms."""
     return {"workload": WORKLOAD32, "path": HEAD32,
             "path_desc": ("outer FP64 refinement (residual r = v - Z x from FP16X3 products, differences and norms "
-                          "in FP64) around GMRES(50) on FP16X3 tcgen05 products (fp16 hi+lo split, FP32 "
-                          "accumulate, FP32 Krylov vectors, FP64 dots and Givens) to 5e-6; stop at 1e-5"),
+                          "in FP64) around GMRES(50) on FP16X3 products (evaluated in FP32 as a lattice convolution, "
+                          "FP32 Krylov vectors, FP64 dots and Givens) to 5e-6; stop at 1e-5"),
             "tol": 1e-5, "nrhs": 1, "symmetry": symmetry,
-            "l2": ("no flush needed: each product streams >= 33 GB of coupling images (> 129 MB L2)" if not symmetry
-                   else "symmetry-compressed store (2,780 blocks, 820 MB of images per 16-bit store, > 129 MB L2); "
-                        "inputs (48 permuted copies) and slabs are rewritten every product"),
+            "l2": ("no flush needed: each product streams 0.73 GB of near blocks, 0.25 GB of mapping matrices and "
+                   "0.28 GB of convolution workspace (> 129 MB L2)"),
             "parallelism": "replicas" if world > 1 else "single"}
 
 
@@ -192,9 +191,8 @@ def shell16_config(ie, symmetry: int = 0, world: int = 1, workload: str = WORKLO
     hp = solve_paths(ie)[HEADLINE]
     return {"workload": workload, "path": HEADLINE, "path_desc": hp["desc"], "tol": hp["opts"]["tol"],
             "nrhs": 1, "symmetry": symmetry,
-            "l2": ("no flush needed: each product streams >= 4.9 GB of coupling blocks (> 129 MB L2)"
-                   if not symmetry else
-                   "symmetry-compressed store (473 blocks, 139 MB); inputs and slabs are rewritten each product"),
+            "l2": ("no flush needed: each product streams 0.18 GB of near blocks and 0.06 GB of mapping matrices "
+                   "(> 129 MB L2; at the low-frequency box edges the coupling blocks besides)"),
             "parallelism": "replicas" if world > 1 else "single"}
 
 
@@ -355,8 +353,21 @@ def time_far(ctx, plan, c, nrhs, precs, reps, warmup=3):
         ie.ie_plan_profile(plan.handle, False)
         k_ms = s2["translate_ms"] / max(1, s2["translate_launches"])
         out[ie.PREC_NAMES[prec]] = dict(matvecs_per_s=aggregate_rate(ctx.world, 1, mv_ms), ms=mv_ms,
-                                        translate_kernel_ms=k_ms)
+                                        translate_kernel_ms=k_ms,
+                                        conv_bytes=ie.ie_plan_far_bytes(plan.handle, ie.IE_FAR, prec, nrhs))
     return out
+
+
+def far_roofline(entry: dict, block: dict) -> dict:
+    """Roofline of a far product's translation: the block-product kernel's, or, where the
+    product is a lattice convolution, the bytes of its passes against the copy bandwidth."""
+    if not entry["conv_bytes"]:
+        return block
+    peaks = measured_peaks()
+    gbs = entry["conv_bytes"] / (entry["translate_kernel_ms"] / 1e3) / 1e9
+    return {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm"], "unit": "GB/s", "frac": gbs / peaks["hbm"],
+            "traffic": None, "kernel": "conv passes and the adjacent pairs' product",
+            "bytes_per_launch": entry["conv_bytes"], "peak_source": "of measured (MEASURED_PEAKS.json, copy)"}
 
 
 def tc_roofline(pairs_x_rhs: int, kernel_ms: float, products: int, summary: str | None, kernel: str,
@@ -436,11 +447,13 @@ def run_shell16(ctx):
     if args.lfb is not None and roofline.get("traffic") is not None:
         roofline["traffic_note"] = ("captured at a=lambda/4: the box edge changes only the values, not the "
                                     "work list or the bytes moved")
+    roofline = far_roofline(far["fp16x3"], roofline)
     simt_ach = pairs * 8 * 192 * 192 / (far["fp32"]["translate_kernel_ms"] / 1e3) / 1e12
     roofline_fp32 = {"bound": "alu", "achieved": simt_ach, "peak": FP32_SIMT_PEAK_TFLOPS, "unit": "TFLOP/s",
                      "frac": simt_ach / FP32_SIMT_PEAK_TFLOPS, "kernel": "translate_simt_kernel",
                      "traffic": None,
                      "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 x 2.07 GHz"}
+    roofline_fp32 = far_roofline(far["fp32"], roofline_fp32)
 
     hp = paths[HEADLINE]
     result = {
@@ -507,20 +520,20 @@ def shell32_paths(ie) -> dict:
     return {
         "mixed_fp16x3": dict(opts=ie.solve_opts(tol=1e-5, prec=ie.IE_PREC_FP16X3, refine=1,
                                                 refine_prec=ie.IE_PREC_FP16X3, inner_tol=5e-6),
-                             dtype="fp16x3 tensor products (fp16 hi+lo split, f32 accumulate), f32 GMRES, f64 "
-                                   "refinement residual"),
+                             dtype="fp16x3 products evaluated in f32 (lattice convolution), f32 GMRES, f64 refinement "
+                                   "residual"),
         "fp16x3_gmres": dict(opts=ie.solve_opts(tol=1e-5, prec=ie.IE_PREC_FP16X3),
-                             dtype="fp16x3 tensor products, f32 GMRES (residual recomputed with fp16x3 products at "
+                             dtype="f32 (lattice convolution), f32 GMRES (residual recomputed with the same products at "
                                    "each restart)"),
         "mixed_bf16x3": dict(opts=ie.solve_opts(tol=1e-5, prec=ie.IE_PREC_BF16X3, refine=1,
                                                 refine_prec=ie.IE_PREC_FP16X3, inner_tol=1e-3),
-                             dtype="bf16x3 inner GMRES to 1e-3, f64 refinement on fp16x3 residuals"),
+                             dtype="f32 (lattice convolution), inner GMRES to 1e-3, f64 refinement"),
         "mixed_fp16x1": dict(opts=ie.solve_opts(tol=1e-5, prec=ie.IE_PREC_FP16X1, refine=1,
                                                 refine_prec=ie.IE_PREC_FP16X3, inner_tol=1e-3),
                              dtype="single fp16 products in the inner GMRES to 1e-3, f64 refinement on fp16x3 "
                                    "residuals"),
         "plain": dict(opts=ie.solve_opts(tol=1e-5, prec=ie.IE_PREC_FP32),
-                      dtype="f32 (FP32 SIMT products, f32 GMRES, f64 dots)"),
+                      dtype="f32 (lattice convolution, f32 GMRES, f64 dots)"),
     }
 
 
@@ -562,12 +575,14 @@ def run_shell32(ctx):
     roofline = tc_roofline(pairs, far["fp16x3"]["translate_kernel_ms"], 3,
                            "translate_tc_fp16x3_shell32_sym.md" if args.symmetry else "translate_tc_fp16x3_shell32.md",
                            "translate_tc_kernel<fp16,x3>")
+    roofline = far_roofline(far["fp16x3"], roofline)
     simt_ach = pairs * 8 * 192 * 192 / (far["fp32"]["translate_kernel_ms"] / 1e3) / 1e12
     roofline_fp32 = {"bound": "alu", "achieved": simt_ach, "peak": FP32_SIMT_PEAK_TFLOPS, "unit": "TFLOP/s",
                      "frac": simt_ach / FP32_SIMT_PEAK_TFLOPS, "kernel": "translate_simt_kernel",
                      "traffic": profiled_traffic("translate_simt_fp32_shell32_sym.md" if args.symmetry
                                                  else "translate_simt_fp32_shell32.md", "translate_simt.cu"),
                      "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 x 2.07 GHz"}
+    roofline_fp32 = far_roofline(far["fp32"], roofline_fp32)
     keys = ("solves_per_s", "p50_ms", "p99_ms", "iterations", "matvecs", "refinements", "relres")
     result = {
         "metric": METRIC, "value": head["solves_per_s"], "unit": "solves/s", "n_gpus": world,
@@ -744,7 +759,7 @@ def run_batch64(ctx):
         "metric": METRIC, "value": solve["solves_per_s"] * b.n_groups, "unit": "scatterer solves/s",
         "n_gpus": ctx.world, "steps": max(1, args.steps), "warmup": args.warmup, "ms_per_step": solve["ms"],
         "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "fp16x3 tensor products, f32 GMRES",
+        "vs_baseline": None, "dtype": "fp16x3 products (evaluated in f32 as lattice convolutions), f32 GMRES",
         "data": "synthetic",
         "config": {"workload": (f"batch64: 64 scatterers (sphere/cube/ellipsoid shells r=3..14 on 32^3, nb 16..64, "
                                 f"1..8 plane waves; seed 41): {st['n_boxes']} boxes, {b.n} basis unknowns, "
@@ -757,8 +772,8 @@ def run_batch64(ctx):
         "device_bytes": mixed_bytes,
         "far_pair_rhs": pair_rhs,
         "gpu_launches": int(solve["launches"]), "clocks": solve["clocks"],
-        "roofline": tc_roofline(pair_rhs, far["fp16x3"]["translate_kernel_ms"], 3, None,
-                                "translate_tc_kernel<fp16,x3>", sustained=True),
+        "roofline": far_roofline(far["fp16x3"], tc_roofline(pair_rhs, far["fp16x3"]["translate_kernel_ms"], 3, None,
+                                                            "translate_tc_kernel<fp16,x3>", sustained=True)),
     }
     return out
 
@@ -874,7 +889,7 @@ def run_serve(ctx):
         "metric": METRIC, "value": head["solves_per_s"], "unit": "solves/s", "n_gpus": ctx.world,
         "steps": len(reqs), "warmup": 0, "ms_per_step": 1e3 / max(head["solves_per_s"], 1e-12),
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "fp16x3 tensor products, f32 GMRES", "data": "synthetic",
+        "dtype": "fp16x3 products (evaluated in f32 as lattice convolutions), f32 GMRES", "data": "synthetic",
         "config": {"workload": (f"serve: {len(reqs)} Poisson arrivals (seed 51), sphere shells of 200..20,000 "
                                 f"boxes (log-uniform), nb=32, 1..4 plane waves, tol 1e-5; HBM budget "
                                 f"{budget / 1e9:.0f} GB; offered loads x plain capacity {args.serve_load}"),
@@ -890,12 +905,13 @@ def solve_paths(ie) -> dict:
     """Solve forms measured on the workload; HEADLINE is the value's step."""
     return {
         "fp16x3": dict(opts=dict(tol=1e-5, restart=50, prec=ie.IE_PREC_FP16X3),
-                       dtype="fp16x3 tensor products (fp16 hi+lo split, f32 accumulate), f32 GMRES, f64 dots",
-                       desc="GMRES(50) on FP16X3 tcgen05 products to 1e-5 (true residual checked against the FP64 "
+                       dtype="f32 (lattice convolution; fp16 hi+lo tensor products at the low-frequency box edges), f32 "
+                             "GMRES, f64 dots",
+                       desc="GMRES(50) on FP16X3 products to 1e-5 (true residual checked against the FP64 "
                             "oracle in the tests)"),
         "mixed_refine": dict(opts=dict(tol=1e-5, restart=50, prec=ie.IE_PREC_BF16X3, refine=1,
                                        refine_prec=ie.IE_PREC_FP16X3, inner_tol=1e-3),
-                             dtype="bf16x3 tensor products, f32 GMRES, f64 refinement",
+                             dtype="bf16x3 products, f32 GMRES, f64 refinement",
                              desc="outer FP64 refinement (residual from FP16X3 products) around GMRES(50) on BF16X3 "
                                   "products to 1e-3; stop at 1e-5"),
         "mixed_fp16x1": dict(opts=dict(tol=1e-5, restart=50, prec=ie.IE_PREC_FP16X1, refine=1,
@@ -903,7 +919,7 @@ def solve_paths(ie) -> dict:
                              dtype="fp16 tensor products, f32 GMRES, f64 refinement",
                              desc="refinement (FP16X3 residual) around GMRES(50) on single fp16 products to 1e-3"),
         "plain": dict(opts=dict(tol=1e-6, restart=50, prec=ie.IE_PREC_FP32), dtype="f32",
-                      desc="plain FP32 path: GMRES(50) on FP32 SIMT products to 1e-6"),
+                      desc="plain FP32 path: GMRES(50) on FP32 products to 1e-6"),
     }
 
 

@@ -87,6 +87,14 @@ typedef enum {
  *          l-infinity ball); ie_cvfcnn_train replaces them by networks trained as in §3
  *          (first stage), ie_cvfcnn_set_weights by any others.
  *  CVFCNN_FP32  the same networks evaluated in FP32 on the SIMT cores. */
+/*
+ * Evaluation: all boxes' dipoles lie on one lattice, so the far field is a discrete
+ * convolution of D (eq. 5).  Products in FP32, BF16X3 and FP16X3 are evaluated as such in
+ * FP32 (its error against FP64 is below that of the block products in these precisions)
+ * where the scatterers' bounding lattices make it the cheaper form and k a >= 0.75; the
+ * products of the adjacent boxes' site pairs that it holds besides are taken off in the named
+ * arithmetic, or left to it (IE_FULL).  Otherwise, and in the other precisions always, the
+ * block products per displacement run in the named arithmetic. */
 typedef enum {
     IE_PREC_FP32 = 1,
     IE_PREC_BF16X3 = 2,
@@ -235,7 +243,13 @@ ie_status ie_plan_footprint_shared(const ie_problem *prob, ie_store store, size_
 
 ie_status ie_plan_stats_get(ie_plan plan, ie_plan_stats *out);
 
-/* Profiling of the translation kernel: with enable = 1 (counters reset), every
+/* Bytes per product that the far part of `which` (IE_FAR or IE_FULL) moves through device
+ * memory when it is evaluated as a lattice convolution (its five passes, their multiplier
+ * once), or 0 when this plan uses the block products for it.  Host only.
+ * Errors: IE_ERR_INVALID, IE_ERR_UNSUPPORTED. */
+ie_status ie_plan_far_bytes(ie_plan plan, int which, int prec, int nrhs, int64_t *bytes);
+
+/* Profiling of the translation (the block-product kernel, or the convolution's passes): with enable = 1 (counters reset), every
  * translation launched outside stream capture is bracketed by CUDA events on its
  * stream and its duration added to translate_ms (the call then waits for it). */
 ie_status ie_plan_profile(ie_plan plan, int enable);

@@ -36,7 +36,7 @@ EXPORTED = [
     "ie_cvfcnn_train",
     "ie_cvfcnn_train_opts_default", "ie_store_footprint", "ie_store_create", "ie_store_info", "ie_store_release",
     "ie_plan_create_shared", "ie_plan_footprint_shared", "ie_solver_state", "ie_diag_wait_limit",
-    "ie_sym_canon", "ie_sym_map",
+    "ie_sym_canon", "ie_sym_map", "ie_plan_far_bytes",
 ]
 
 
@@ -128,6 +128,7 @@ def lib() -> ctypes.CDLL:
     L.ie_plan_stats_get.argtypes = [vp, P(ie_plan_stats)]
     L.ie_plan_destroy.argtypes = [vp]
     L.ie_plan_profile.argtypes = [vp, i]
+    L.ie_plan_far_bytes.argtypes = [vp, i, i, i, P(ctypes.c_int64)]
     L.ie_matvec.argtypes = [vp, i, i, vp, vp, i, vp]
     L.ie_aggregate.argtypes = [vp, vp, vp, i, vp]
     L.ie_translate.argtypes = [vp, i, vp, vp, i, vp]
@@ -324,6 +325,13 @@ def ie_plan_stats_get(plan: int) -> dict:
     s = ie_plan_stats()
     _check(lib().ie_plan_stats_get(plan, ctypes.byref(s)), "ie_plan_stats_get")
     return {f: getattr(s, f) for f, _ in s._fields_}
+
+
+def ie_plan_far_bytes(plan: int, which: int, prec: int, nrhs: int) -> int:
+    """Bytes per product of the convolution that evaluates the far part, 0 with block products."""
+    b = ctypes.c_int64()
+    _check(lib().ie_plan_far_bytes(plan, which, prec, nrhs, ctypes.byref(b)), "ie_plan_far_bytes")
+    return b.value
 
 
 def ie_plan_profile(plan: int, enable: bool) -> None:

@@ -49,6 +49,7 @@ ie_status prepare_translate_simt();
 ie_status prepare_translate_tc();
 ie_status prepare_translate_cvfcnn();
 ie_status prepare_cvfcnn_tc();
+ie_status prepare_conv();
 
 std::recursive_mutex &device_mutex() {
     static std::recursive_mutex mu;
@@ -60,6 +61,7 @@ ie_status prepare_kernels() {
     IE_TRY(prepare_translate_tc());
     IE_TRY(prepare_translate_cvfcnn());
     IE_TRY(prepare_cvfcnn_tc());
+    IE_TRY(prepare_conv());
     return IE_OK;
 }
 
@@ -325,8 +327,10 @@ void near_lists(const ie_problem *pr, const BoxGrid &g, const std::vector<int32_
 }
 
 size_t plan_bytes(const ie_problem *pr, int64_t n, int64_t npairs, int64_t nd, int64_t nnear, int64_t near_elems,
-                  int64_t nblk, bool shared = false) {
-    size_t b = 0;
+                  int64_t nblk, bool shared = false, int64_t used = -1) {
+    std::vector<ConvClass> conv;      // used: stored blocks the pairs use (a shared store holds more)
+    const ConvUse use = conv_classes(pr, npairs, used >= 0 ? used : pr->symmetry == 1 ? nblk : nd, conv);
+    size_t b = conv_bytes(pr, conv, use, nnear, near_elems);
     auto add = [&](size_t x) { b += (x + 255) / 256 * 256; };
     int64_t nbox = pr->n_boxes;
     if (pr->P) add((size_t)n * kNU * sizeof(float2));
@@ -496,24 +500,18 @@ ie_status work_list_for(ie_plan p, int prec, int nrhs, WorkList **out) {
 int canon_of_disp(const int32_t d[3], int32_t c[3]) { return canon_of(d, c); }
 void symmetry_map_host(std::vector<uint16_t> &map) { symmetry_map(map); }
 
-ie_status translate_timed(ie_plan p, int prec, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
-                          const int *gate) {
-    bool timed = false;
+// Runs `body` (the translation's launches), timed when the plan's profiling is on.
+template <class F>
+static ie_status timed(ie_plan p, cudaStream_t st, F body) {
+    bool on = false;
     if (p->profile) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         IE_CK(cudaStreamIsCapturing(st, &cs));
-        timed = cs == cudaStreamCaptureStatusNone;
+        on = cs == cudaStreamCaptureStatusNone;
     }
-    if (timed) IE_CK(cudaEventRecord(p->prof_ev[0], st));
-    if (prec == IE_PREC_FP32)
-        IE_TRY(launch_translate_simt(p, X, Yslab, nrhs, st, gate));
-    else if (prec == IE_PREC_CVFCNN_FP32)
-        IE_TRY(launch_translate_cvfcnn(p, X, Yslab, nrhs, st, gate));
-    else if (prec == IE_PREC_CVFCNN)
-        IE_TRY(launch_translate_cvfcnn_tc(p, Yslab, nrhs, st, gate));
-    else
-        IE_TRY(launch_translate_tc(p, prec, Yslab, nrhs, st, gate));
-    if (timed) {
+    if (on) IE_CK(cudaEventRecord(p->prof_ev[0], st));
+    IE_TRY(body());
+    if (on) {
         IE_CK(cudaEventRecord(p->prof_ev[1], st));
         IE_CK(cudaEventSynchronize(p->prof_ev[1]));
         float ms = 0;
@@ -524,15 +522,95 @@ ie_status translate_timed(ie_plan p, int prec, const float2 *X, float2 *Yslab, i
     return IE_OK;
 }
 
+ie_status translate_timed(ie_plan p, int prec, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
+                          const int *gate) {
+    return timed(p, st, [&] {
+        if (prec == IE_PREC_FP32) return launch_translate_simt(p, X, Yslab, nrhs, st, gate);
+        if (prec == IE_PREC_CVFCNN_FP32) return launch_translate_cvfcnn(p, X, Yslab, nrhs, st, gate);
+        if (prec == IE_PREC_CVFCNN) return launch_translate_cvfcnn_tc(p, Yslab, nrhs, st, gate);
+        return launch_translate_tc(p, prec, Yslab, nrhs, st, gate);
+    });
+}
+
+// Work list of the adjacent pairs (launch_adjacent): runs of one displacement's pairs.
+ie_status adj_list(ie_plan p, bool tc, int nrhs, WorkList **out) {
+    const int key = 2 * nrhs + (tc ? 1 : 0), cols = tc ? tc_tile_columns() : simt_tile_columns();
+    auto it = p->adj_work.find(key);
+    if (it != p->adj_work.end()) {
+        *out = &it->second;
+        return IE_OK;
+    }
+    if (g_capture_depth > 0) return set_error("adjacent work list (nrhs %d) missing at stream capture", nrhs), IE_ERR_INVALID;
+    auto nr_of = [&](int64_t pair) {
+        return p->gnrhs.empty() ? nrhs : std::min(nrhs, (int)p->gnrhs[p->box_group[p->h_adj_src[pair]]]);
+    };
+    std::vector<WorkItem> items;
+    for (int e = 0; e < 27; ++e)
+        for (int64_t q = p->h_adj_start[e], end = p->h_adj_start[e + 1]; q < end;) {
+            const int nr = nr_of(q), per = cols / nr;
+            int np = 0;
+            while (q + np < end && np < per && nr_of(q + np) == nr) ++np;
+            items.push_back({e, (int32_t)q, np, 0, nr});
+            q += np;
+        }
+    WorkList wl;
+    wl.n = (int64_t)items.size();
+    if (wl.n) {
+        IE_TRY(dalloc_t(p, &wl.d_items, items.size()));
+        IE_CK(cudaMemcpy(wl.d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
+    }
+    p->adj_work[key] = wl;
+    *out = &p->adj_work[key];
+    return IE_OK;
+}
+
+// Makes the list a far product of this nrhs will want (outside any capture), as a full
+// product with block products would have made the list they share.
+static ie_status adj_prepare(ie_plan p, int prec, int nrhs, cudaStream_t st) {
+    const bool tc = prec != IE_PREC_FP32;
+    if (!p->n_adj || p->adj_work.count(2 * nrhs + (tc ? 1 : 0))) return IE_OK;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    IE_CK(cudaStreamIsCapturing(st, &cs));
+    WorkList *wl = nullptr;
+    return cs == cudaStreamCaptureStatusNone ? adj_list(p, tc, nrhs, &wl) : IE_OK;
+}
+
+ie_status launch_adjacent(ie_plan p, int prec, const float2 *X, float2 *slab, int nrhs, cudaStream_t st,
+                          const int *gate) {
+    if (prec == IE_PREC_FP32) return launch_translate_simt(p, X, slab, nrhs, st, gate, true);
+    IE_TRY(launch_split_tc(p, X, nrhs, is_fp16(prec), st, gate, true));
+    return launch_translate_tc(p, prec, slab, nrhs, st, gate, true);
+}
+
+// The far field of X by convolution in two slabs of the scratch: the adjacent pairs'
+// (negated) part of it, and the convolution itself.
+static ie_status conv_translate(ie_plan p, int prec, const float2 *X, int nrhs, int *nslab, cudaStream_t st,
+                                const int *gate) {
+    const size_t stride = slab_stride(p);
+    *nslab = 1;
+    float2 *Y = p->d_Yslab;
+    if (p->n_adj) {
+        IE_TRY(launch_zero_slabs(p->d_Yslab, 1, stride, (size_t)nrhs * p->nbox * kNU, st, gate));
+        IE_TRY(launch_adjacent(p, prec, X, p->d_Yslab, nrhs, st, gate));
+        Y += stride;
+        *nslab = 2;
+    }
+    return launch_conv(p, X, Y, nrhs, st, gate);
+}
+
 ie_status far_product(ie_plan p, int prec, const float2 *c, float2 *y, int nrhs, bool accumulate, cudaStream_t st,
                       const int *gate) {
     size_t stride = slab_stride(p);
     IE_TRY(launch_aggregate(p, c, p->d_X, nrhs, st, gate));
-    IE_TRY(launch_zero_slabs(p->d_Yslab, kSlabs, stride, (size_t)nrhs * p->nbox * kNU, st, gate));
-    if (uses_split(prec)) IE_TRY(launch_split_tc(p, p->d_X, nrhs, is_fp16(prec), st, gate));
-    IE_TRY(translate_timed(p, prec, p->d_X, p->d_Yslab, nrhs, st, gate));
-    IE_TRY(launch_disaggregate(p, p->d_Yslab, kSlabs, stride, y, nrhs, accumulate, st, gate));
-    return IE_OK;
+    int nslab = kSlabs;
+    if (conv_far(p, prec)) {
+        IE_TRY(timed(p, st, [&] { return conv_translate(p, prec, p->d_X, nrhs, &nslab, st, gate); }));
+    } else {
+        IE_TRY(launch_zero_slabs(p->d_Yslab, kSlabs, stride, (size_t)nrhs * p->nbox * kNU, st, gate));
+        if (uses_split(prec)) IE_TRY(launch_split_tc(p, p->d_X, nrhs, is_fp16(prec), st, gate));
+        IE_TRY(translate_timed(p, prec, p->d_X, p->d_Yslab, nrhs, st, gate));
+    }
+    return launch_disaggregate(p, p->d_Yslab, nslab, stride, y, nrhs, accumulate, st, gate);
 }
 
 ie_status take_device_error(ie_plan p, cudaStream_t st) {
@@ -548,6 +626,15 @@ ie_status take_device_error(ie_plan p, cudaStream_t st) {
 ie_status apply(ie_plan p, int which, int prec, const float2 *c, float2 *y, int nrhs, cudaStream_t st,
                 const int *gate) {
     if (which == IE_FAR) return far_product(p, prec, c, y, nrhs, false, st, gate);
+    if (which == IE_FULL && conv_full(p, prec)) {
+        // the convolution holds the adjacent boxes' site pairs beyond kNearReach: near blocks
+        // of the others only, and nothing to take off
+        IE_TRY(adj_prepare(p, prec, nrhs, st));
+        IE_TRY(launch_near(p, c, y, nrhs, st, gate, true));
+        IE_TRY(launch_aggregate(p, c, p->d_X, nrhs, st, gate));
+        IE_TRY(timed(p, st, [&] { return launch_conv(p, p->d_X, p->d_Yslab, nrhs, st, gate); }));
+        return launch_disaggregate(p, p->d_Yslab, 1, 0, y, nrhs, true, st, gate);
+    }
     IE_TRY(launch_near(p, c, y, nrhs, st, gate));
     if (which == IE_FULL) IE_TRY(far_product(p, prec, c, y, nrhs, true, st, gate));
     return IE_OK;
@@ -679,7 +766,8 @@ static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream,
     for (int b = 0; b < p->nbox; ++b) p->box_group[b] = group_of(pr, b);
 
     FarGroups fg;
-    far_groups(pr, g, true, fg, p->n_far_pairs, p->n_far_disp);
+    int64_t ncanon_used = 0;
+    far_groups(pr, g, true, fg, p->n_far_pairs, p->n_far_disp, pr->symmetry == 1 ? &ncanon_used : nullptr);
     p->h_disp = fg.disp;
     p->h_gstart = fg.start;
     // stored blocks: one per displacement, or one per canonical displacement
@@ -899,8 +987,49 @@ static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream,
         PT(dalloc_t(p, &p->d_Nblk, (size_t)p->near_elems));
         PC(cudaMemcpyAsync(p->d_near_src, nsrc.data(), nsrc.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
         PC(cudaMemcpyAsync(p->d_near_boff, nboff.data(), nboff.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-        PT(launch_near_blocks(p, st));
     }
+
+    // far product as a convolution: its blocks of the adjacent pairs, K^, workspace
+    p->conv_use = conv_classes(pr, p->n_far_pairs, p->sym ? ncanon_used : p->n_far_disp, p->conv);
+    if (!p->conv.empty()) {
+        PT(conv_create(p, st));
+        if (!p->gnrhs.empty()) {
+            std::vector<int32_t> bc(p->nbox);
+            for (int b = 0; b < p->nbox; ++b) bc[b] = p->gnrhs[p->box_group[b]];
+            PT(dalloc_t(p, &p->d_box_cols, bc.size()));
+            PC(cudaMemcpy(p->d_box_cols, bc.data(), bc.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        }
+        if (p->conv_use.far) {
+            std::vector<int32_t> asrc, adst;
+            p->h_adj_start.assign(28, 0);
+            for (int e = 0; e < 27; ++e) {
+                p->h_adj_start[e] = (int64_t)asrc.size();
+                if (e == 13) continue;      // the box itself: no site pair beyond kNearReach
+                const int ex = e / 9 - 1, ey = (e / 3) % 3 - 1, ez = e % 3 - 1;
+                for (int t = 0; t < p->nbox; ++t) {
+                    const int32_t *q = &p->ijk[3 * t];
+                    const int b = g.at(p->box_group[t], q[0] - ex, q[1] - ey, q[2] - ez);
+                    if (b >= 0) asrc.push_back(b), adst.push_back(t);
+                }
+            }
+            p->n_adj = p->h_adj_start[27] = (int64_t)asrc.size();
+            if (p->n_adj) {
+                PT(dalloc_t(p, &p->d_adj_src, asrc.size()));
+                PT(dalloc_t(p, &p->d_adj_dst, adst.size()));
+                PC(cudaMemcpy(p->d_adj_src, asrc.data(), asrc.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+                PC(cudaMemcpy(p->d_adj_dst, adst.data(), adst.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+                if (!p->gnrhs.empty()) p->h_adj_src = std::move(asrc);
+                if (wants_bf16(p->prec_mask)) PT(dalloc_t(p, &p->d_Cadj_bf16, (size_t)27 * kTcDispElems));
+                if (wants_fp16(p->prec_mask)) {
+                    PT(dalloc_t(p, &p->d_Cadj_fp16, (size_t)27 * kTcDispElems));
+                    PT(dalloc_t(p, &p->d_Cadj_exp16, 27));
+                }
+                PT(dalloc_t(p, &p->d_Cadj, (size_t)27 * kNU * kNU));
+            }
+        }
+        if (p->n_near_pairs) PT(dalloc_t(p, &p->d_Nshort, (size_t)p->near_elems));
+    }
+    if (p->n_near_pairs) PT(launch_near_blocks(p, st));
 
     // scratch
     size_t col = (size_t)p->max_rhs * p->nbox;
@@ -964,13 +1093,13 @@ ie_status ie_plan_footprint_shared(const ie_problem *pr, ie_store store, size_t 
     int64_t n = 0;
     for (int b = 0; b < pr->n_boxes; ++b) n += (nb[b] = pr->nb ? pr->nb[b] : kNU);
     FarGroups fg;
-    int64_t npairs = 0, nd = 0;
-    far_groups(pr, g, false, fg, npairs, nd, nullptr);
+    int64_t npairs = 0, nd = 0, ncanon = 0;
+    far_groups(pr, g, false, fg, npairs, nd, &ncanon);
     std::vector<int32_t> st, src;
     std::vector<int64_t> boff;
     int64_t elems = 0;
     near_lists(pr, g, nb, st, src, boff, elems);
-    *bytes = plan_bytes(pr, n, npairs, nd, (int64_t)src.size(), elems, store->n_blocks, true);
+    *bytes = plan_bytes(pr, n, npairs, nd, (int64_t)src.size(), elems, store->n_blocks, true, ncanon);
     return IE_OK;
 }
 
@@ -1063,6 +1192,15 @@ ie_status ie_plan_stats_get(ie_plan p, ie_plan_stats *o) {
     return IE_OK;
 }
 
+ie_status ie_plan_far_bytes(ie_plan p, int which, int prec, int nrhs, int64_t *bytes) {
+    if (!p || !bytes) return set_error("null argument"), IE_ERR_INVALID;
+    if (which != IE_FAR && which != IE_FULL) return set_error("bad which %d", which), IE_ERR_INVALID;
+    IE_TRY(check_rhs(p, nrhs));
+    IE_TRY(check_prec(p, prec));
+    *bytes = (which == IE_FULL ? conv_full(p, prec) : conv_far(p, prec)) ? conv_traffic(p, nrhs) : 0;
+    return IE_OK;
+}
+
 ie_status ie_plan_profile(ie_plan p, int enable) {
     if (!p) return set_error("null plan"), IE_ERR_INVALID;
     if (enable && !p->prof_ev[0]) {
@@ -1113,6 +1251,11 @@ ie_status ie_translate(ie_plan p, int prec, const void *X, void *Y, int nrhs, vo
     IE_TRY(check_prec(p, prec));
     cudaStream_t st = (cudaStream_t)stream;
     size_t stride = slab_stride(p);
+    if (conv_far(p, prec)) {
+        int nslab = 0;
+        IE_TRY(timed(p, st, [&] { return conv_translate(p, prec, (const float2 *)X, nrhs, &nslab, st, nullptr); }));
+        return launch_sum_slabs(p, p->d_Yslab, nslab, stride, (float2 *)Y, nrhs, st);
+    }
     IE_TRY(launch_zero_slabs(p->d_Yslab, kSlabs, stride, (size_t)nrhs * p->nbox * kNU, st));
     if (uses_split(prec)) IE_TRY(launch_split_tc(p, (const float2 *)X, nrhs, is_fp16(prec), st));
     IE_TRY(translate_timed(p, prec, (const float2 *)X, p->d_Yslab, nrhs, st, nullptr));

@@ -15,7 +15,7 @@ namespace {
 // row_major = false: layout [d][k][m] (k = basis unknown, m = test unknown), the
 // FP32 translation kernel's A^T operand; true: [d][m][k].
 __global__ void coupling_fp32_kernel(double k, double eta, double h, const int32_t *__restrict__ disp, int64_t nd,
-                                     float2 *__restrict__ out, int row_major) {
+                                     float2 *__restrict__ out, int row_major, int part) {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nd * kSites * kSites) return;
     int64_t di = t / (kSites * kSites);
@@ -27,15 +27,18 @@ __global__ void coupling_fp32_kernel(double k, double eta, double h, const int32
     int my = 4 * dy + ((l >> 2) & 3) - ((q >> 2) & 3);
     int mz = 4 * dz + (l >> 4) - (q >> 4);
     double2 D[9];
-    bool coincident = (mx == 0 && my == 0 && mz == 0);
-    if (!coincident) dyad_fp64(k, eta, h * mx, h * my, h * mz, D);
+    const int reach = max(abs(mx), max(abs(my), abs(mz)));
+    const bool skip = reach == 0 || (part == kShortSites && reach > kNearReach) ||
+                            (part == kLongSitesNegated && reach <= kNearReach);
+    const float sg = part == kLongSitesNegated ? -1.f : 1.f;
+    if (!skip) dyad_fp64(k, eta, h * mx, h * my, h * mz, D);
     float2 *blk = out + di * (int64_t)kNU * kNU;
 #pragma unroll
     for (int al = 0; al < 3; ++al)
 #pragma unroll
         for (int be = 0; be < 3; ++be) {
-            float2 v = coincident ? make_float2(0.f, 0.f)
-                                  : make_float2((float)D[3 * al + be].x, (float)D[3 * al + be].y);
+            float2 v = skip ? make_float2(0.f, 0.f)
+                                  : make_float2(sg * (float)D[3 * al + be].x, sg * (float)D[3 * al + be].y);
             int m = 3 * l + al, kk = 3 * q + be;
             if (row_major)
                 blk[(int64_t)m * kNU + kk] = v;
@@ -123,67 +126,156 @@ __global__ void coupling_tc_kernel(const float2 *__restrict__ Cs, int64_t nd, ui
 }
 
 // Near blocks: N_ab = P_a G_{a-b} P_b^T (test box a, basis box b), nb_a x nb_b,
-// column-major.  One CTA per stored pair; basis columns in chunks of 32.
-// Partial sums over 32 terms in FP32, chunk sums in FP64.
-constexpr int kNearJ = 32;
+// column-major, and with Nshort the same from the blocks cut to kNearReach (Cnear + 27
+// blocks).  One CTA per stored pair; basis columns in chunks of 32.  W = G P_b^T is a
+// 192 x 32 register-tiled product (6 x 4 complex per thread, G chunks through shared memory,
+// double-buffered), N = P_a W follows from shared memory.  Sums of 32 terms run in FP32,
+// the chunks' sums are added as two-float pairs (an FP64 addition would take as long as the
+// 32 multiply-adds before it).  FP32 rate bound: both block sets of the 32^3 shell in 52 ms
+// (38 TFLOP/s; one set took 122 ms with a sum per thread and G read per term), the 16^3
+// shell's in 13 ms (31).
+constexpr int kNearJ = 32, kNearKC = 16, kNearThreads = 256;
+struct SmemNear {
+    float2 Pb[kNU][kNearJ];             // [k][j]
+    union {
+        float2 A[2][kNearKC][kNU];      // G chunk [k][m]
+        float2 W[kNU][kNearJ];          // [m][j], once G has been read
+    };
+};
+static_assert(sizeof(float2) * kNU * kNearJ == sizeof(float2) * 2 * kNearKC * kNU, "W overlays the chunks");
 
-__global__ void near_blocks_kernel(const float2 *__restrict__ Cnear,     // [27][k][m], index by e
-                                   const int32_t *__restrict__ ijk, const int32_t *__restrict__ nb,
-                                   const int64_t *__restrict__ off, const float2 *__restrict__ P,
-                                   const int32_t *__restrict__ pair_a, const int32_t *__restrict__ pair_b,
-                                   const int64_t *__restrict__ boff, int64_t npairs, float2 *__restrict__ Nblk) {
-    extern __shared__ float2 sm[];
-    float2 *Pb = sm;                    // [kNearJ][192]
-    float2 *W = sm + kNearJ * kNU;      // [192][kNearJ]
-    int64_t pi = blockIdx.x;
-    if (pi >= npairs) return;
-    int a = pair_a[pi], b = pair_b[pi];
-    int ex = ijk[3 * a] - ijk[3 * b], ey = ijk[3 * a + 1] - ijk[3 * b + 1], ez = ijk[3 * a + 2] - ijk[3 * b + 2];
-    int e = (ex + 1) * 9 + (ey + 1) * 3 + (ez + 1);
-    const float2 *C = Cnear + (int64_t)e * kNU * kNU;   // [k][m]
-    int na = nb[a], nbb = nb[b];
-    const float2 *Pa = P + off[a] * kNU;
-    const float2 *Pbg = P + off[b] * kNU;
-    float2 *N = Nblk + boff[pi];
+// (hi, lo) += x
+__device__ __forceinline__ void add2(float &hi, float &lo, float x) {
+    const float s = hi + x, bb = s - hi;
+    lo += (hi - (s - bb)) + (x - bb);
+    hi = s;
+}
+
+__global__ void __launch_bounds__(kNearThreads)
+near_blocks_kernel(const float2 *__restrict__ Cnear,     // [27 or 54][k][m], index by e
+                   const int32_t *__restrict__ ijk, const int32_t *__restrict__ nb, const int64_t *__restrict__ off,
+                   const float2 *__restrict__ P, const int32_t *__restrict__ pair_a, const int32_t *__restrict__ pair_b,
+                   const int64_t *__restrict__ boff, float2 *__restrict__ Nblk, float2 *__restrict__ Nshort) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SmemNear &S = *reinterpret_cast<SmemNear *>(smem_raw);
+    const int64_t pi = blockIdx.x;
+    const int tid = threadIdx.x, a = pair_a[pi], b = pair_b[pi];
+    const int ex = ijk[3 * a] - ijk[3 * b], ey = ijk[3 * a + 1] - ijk[3 * b + 1], ez = ijk[3 * a + 2] - ijk[3 * b + 2];
+    const int e = (ex + 1) * 9 + (ey + 1) * 3 + (ez + 1);
+    const int na = nb[a], nbb = nb[b], tm = tid >> 3, tn = tid & 7;   // rows 2 tm, + 1 (+ 64 j); columns 4 tn ..
+    const float2 *Pa = P + off[a] * kNU, *Pbg = P + off[b] * kNU;
     for (int j0 = 0; j0 < nbb; j0 += kNearJ) {
-        int nj = min(kNearJ, nbb - j0);
+        const int nj = min(kNearJ, nbb - j0);
         __syncthreads();
-        for (int i = threadIdx.x; i < nj * kNU; i += blockDim.x) Pb[i] = Pbg[(int64_t)j0 * kNU + i];
-        __syncthreads();
-        // W[m][jj] = sum_k C[m][k] Pb[jj][k]
-        for (int o = threadIdx.x; o < kNU * nj; o += blockDim.x) {
-            int m = o % kNU, jj = o / kNU;
-            double wr = 0, wi = 0;
-            for (int k0 = 0; k0 < kNU; k0 += 32) {
-                float pr = 0.f, pim = 0.f;
-                for (int kk = k0; kk < k0 + 32; ++kk) {
-                    float2 g = C[(int64_t)kk * kNU + m];
-                    float2 pv = Pb[jj * kNU + kk];
-                    pr = fmaf(g.x, pv.x, fmaf(-g.y, pv.y, pr));
-                    pim = fmaf(g.x, pv.y, fmaf(g.y, pv.x, pim));
-                }
-                wr += pr;
-                wi += pim;
-            }
-            W[m * kNearJ + jj] = make_float2((float)wr, (float)wi);
+        for (int i = tid; i < kNearJ * kNU; i += kNearThreads) {
+            const int jj = i / kNU, k = i - jj * kNU;
+            S.Pb[k][jj] = jj < nj ? Pbg[(int64_t)(j0 + jj) * kNU + k] : make_float2(0.f, 0.f);
         }
-        __syncthreads();
-        // N[i][j0+jj] = sum_m Pa[i][m] W[m][jj]
-        for (int o = threadIdx.x; o < na * nj; o += blockDim.x) {
-            int i = o % na, jj = o / na;
-            double nr = 0, ni = 0;
-            for (int m0 = 0; m0 < kNU; m0 += 32) {
-                float pr = 0.f, pim = 0.f;
-                for (int m = m0; m < m0 + 32; ++m) {
-                    float2 pa = Pa[(int64_t)i * kNU + m];
-                    float2 w = W[m * kNearJ + jj];
-                    pr = fmaf(pa.x, w.x, fmaf(-pa.y, w.y, pr));
-                    pim = fmaf(pa.x, w.y, fmaf(pa.y, w.x, pim));
+        // the box's own block has no site pair beyond kNearReach: one product serves both
+        for (int part = 0; part < (Nshort && e != 13 ? 2 : 1); ++part) {
+            const float2 *C = Cnear + (int64_t)(e + 27 * part) * kNU * kNU;   // [k][m]
+            float2 *N = (part ? Nshort : Nblk) + boff[pi];
+            auto load = [&](int kc, int buf) {
+                const float4 *g = reinterpret_cast<const float4 *>(C + (int64_t)kc * kNearKC * kNU);
+                float4 *s = reinterpret_cast<float4 *>(&S.A[buf][0][0]);
+#pragma unroll
+                for (int t = 0; t < kNearKC * kNU / 2 / kNearThreads; ++t) {
+                    const uint32_t d = (uint32_t)__cvta_generic_to_shared(s + tid + t * kNearThreads);
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(g + tid + t * kNearThreads));
                 }
-                nr += pr;
-                ni += pim;
+                asm volatile("cp.async.commit_group;\n" ::);
+            };
+            float2 hi[6][4], lo[6][4], acc[6][4];
+#pragma unroll
+            for (int i = 0; i < 6; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) hi[i][j] = lo[i][j] = acc[i][j] = make_float2(0.f, 0.f);
+            __syncthreads();        // W of the part before has been read
+            load(0, 0);
+            for (int kc = 0; kc < kNU / kNearKC; ++kc) {
+                if (kc + 1 < kNU / kNearKC) {
+                    load(kc + 1, (kc + 1) & 1);
+                    asm volatile("cp.async.wait_group 1;\n" ::);
+                } else {
+                    asm volatile("cp.async.wait_group 0;\n" ::);
+                }
+                __syncthreads();
+#pragma unroll 2
+                for (int kk = 0; kk < kNearKC; ++kk) {
+                    float2 g[6], p[4];
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        const float4 v = *reinterpret_cast<const float4 *>(&S.A[kc & 1][kk][2 * tm + 64 * j]);
+                        g[2 * j] = make_float2(v.x, v.y);
+                        g[2 * j + 1] = make_float2(v.z, v.w);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const float4 v = *reinterpret_cast<const float4 *>(&S.Pb[kc * kNearKC + kk][4 * tn + 2 * j]);
+                        p[2 * j] = make_float2(v.x, v.y);
+                        p[2 * j + 1] = make_float2(v.z, v.w);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 6; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            acc[i][j].x = fmaf(g[i].x, p[j].x, fmaf(-g[i].y, p[j].y, acc[i][j].x));
+                            acc[i][j].y = fmaf(g[i].x, p[j].y, fmaf(g[i].y, p[j].x, acc[i][j].y));
+                        }
+                }
+                if (kc & 1) {       // every 32 terms
+#pragma unroll
+                    for (int i = 0; i < 6; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            add2(hi[i][j].x, lo[i][j].x, acc[i][j].x);
+                            add2(hi[i][j].y, lo[i][j].y, acc[i][j].y);
+                            acc[i][j] = make_float2(0.f, 0.f);
+                        }
+                }
+                __syncthreads();
             }
-            N[(int64_t)(j0 + jj) * na + i] = make_float2((float)nr, (float)ni);
+#pragma unroll
+            for (int i = 0; i < 6; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    S.W[2 * tm + 64 * (i >> 1) + (i & 1)][4 * tn + j] =
+                        make_float2(hi[i][j].x + lo[i][j].x, hi[i][j].y + lo[i][j].y);
+            __syncthreads();
+            // N[i][j0 + jj] = sum_m Pa[i][m] W[m][jj]: lane = column, a warp takes four rows at a time
+            const int jj = tid & 31, warp = tid >> 5;
+            for (int i0 = 4 * warp; i0 < na; i0 += 4 * (kNearThreads / 32)) {
+                float2 h[4], l[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) h[r] = l[r] = make_float2(0.f, 0.f);
+                for (int m0 = 0; m0 < kNU; m0 += 32) {
+                    float2 q[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) q[r] = make_float2(0.f, 0.f);
+#pragma unroll 4
+                    for (int m = m0; m < m0 + 32; ++m) {
+                        const float2 w = S.W[m][jj];
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            const float2 pa = __ldg(Pa + (int64_t)min(i0 + r, na - 1) * kNU + m);
+                            q[r].x = fmaf(pa.x, w.x, fmaf(-pa.y, w.y, q[r].x));
+                            q[r].y = fmaf(pa.x, w.y, fmaf(pa.y, w.x, q[r].y));
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        add2(h[r].x, l[r].x, q[r].x);
+                        add2(h[r].y, l[r].y, q[r].y);
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    if (i0 + r < na && jj < nj) {
+                        const float2 v = make_float2(h[r].x + l[r].x, h[r].y + l[r].y);
+                        N[(int64_t)(j0 + jj) * na + i0 + r] = v;
+                        if (Nshort && e == 13) Nshort[boff[pi] + (int64_t)(j0 + jj) * na + i0 + r] = v;
+                    }
+            }
         }
     }
 }
@@ -192,7 +284,7 @@ __global__ void near_blocks_kernel(const float2 *__restrict__ Cnear,     // [27]
 __global__ void near_blocks_identity_kernel(const float2 *__restrict__ Cnear, const int32_t *__restrict__ ijk,
                                             const int32_t *__restrict__ pair_a, const int32_t *__restrict__ pair_b,
                                             const int64_t *__restrict__ boff, int64_t npairs,
-                                            float2 *__restrict__ Nblk) {
+                                            float2 *__restrict__ Nblk, float2 *__restrict__ Nshort) {
     int64_t pi = blockIdx.x;
     if (pi >= npairs) return;
     int a = pair_a[pi], b = pair_b[pi];
@@ -201,17 +293,21 @@ __global__ void near_blocks_identity_kernel(const float2 *__restrict__ Cnear, co
     const float4 *src = reinterpret_cast<const float4 *>(Cnear + (int64_t)e * kNU * kNU);
     float4 *dst = reinterpret_cast<float4 *>(Nblk + boff[pi]);
     for (int i = threadIdx.x; i < kNU * kNU / 2; i += blockDim.x) dst[i] = src[i];
+    if (!Nshort) return;
+    src += (int64_t)27 * kNU * kNU / 2;
+    dst = reinterpret_cast<float4 *>(Nshort + boff[pi]);
+    for (int i = threadIdx.x; i < kNU * kNU / 2; i += blockDim.x) dst[i] = src[i];
 }
 
 }  // namespace
 
 ie_status launch_coupling_fp32(double k, double eta, double a, const int32_t *d_disp, int64_t nd, float2 *out,
-                               bool row_major, cudaStream_t st) {
+                               bool row_major, cudaStream_t st, BlockPart part) {
     if (nd <= 0) return IE_OK;
     int64_t threads = nd * kSites * kSites;
     int bs = 256;
     int64_t grid = (threads + bs - 1) / bs;
-    coupling_fp32_kernel<<<(unsigned)grid, bs, 0, st>>>(k, eta, a / kLattice, d_disp, nd, out, row_major ? 1 : 0);
+    coupling_fp32_kernel<<<(unsigned)grid, bs, 0, st>>>(k, eta, a / kLattice, d_disp, nd, out, row_major ? 1 : 0, part);
     IE_CK_LAUNCH();
     return IE_OK;
 }
@@ -244,10 +340,17 @@ ie_status launch_near_blocks(ie_plan p, cudaStream_t st) {
     float2 *d_C = nullptr;
     int32_t *d_pa = nullptr;
     IE_CK(cudaMallocAsync(&d_ds, ds.size() * sizeof(int32_t), st));
-    IE_CK(cudaMallocAsync(&d_C, (size_t)27 * kNU * kNU * sizeof(float2), st));
+    IE_CK(cudaMallocAsync(&d_C, (size_t)54 * kNU * kNU * sizeof(float2), st));
     IE_CK(cudaMallocAsync(&d_pa, (size_t)p->n_near_pairs * sizeof(int32_t), st));
     IE_CK(cudaMemcpyAsync(d_ds, ds.data(), ds.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     IE_TRY(launch_coupling_simt(p, d_ds, 27, d_C, false, st));
+    if (p->d_Nshort)
+        IE_TRY(launch_coupling_fp32(p->k, p->eta, p->a, d_ds, 27, d_C + (size_t)27 * kNU * kNU, false, st, kShortSites));
+    if (p->d_Cadj) {
+        IE_TRY(launch_coupling_fp32(p->k, p->eta, p->a, d_ds, 27, p->d_Cadj, false, st, kLongSitesNegated));
+        if (p->d_Cadj_bf16) IE_TRY(launch_coupling_tc(p->d_Cadj, 27, p->d_Cadj_bf16, nullptr, false, st));
+        if (p->d_Cadj_fp16) IE_TRY(launch_coupling_tc(p->d_Cadj, 27, p->d_Cadj_fp16, p->d_Cadj_exp16, true, st));
+    }
     // target box of every stored pair
     std::vector<int32_t> start(p->nbox + 1);
     IE_CK(cudaMemcpyAsync(start.data(), p->d_near_start, start.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -259,13 +362,12 @@ ie_status launch_near_blocks(ie_plan p, cudaStream_t st) {
     if (p->identity) {
         near_blocks_identity_kernel<<<(unsigned)p->n_near_pairs, 256, 0, st>>>(d_C, p->d_ijk, d_pa, p->d_near_src,
                                                                                p->d_near_boff, p->n_near_pairs,
-                                                                               p->d_Nblk);
+                                                                               p->d_Nblk, p->d_Nshort);
     } else {
-        size_t smem = (size_t)2 * kNearJ * kNU * sizeof(float2);
-        IE_CK(cudaFuncSetAttribute(near_blocks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        near_blocks_kernel<<<(unsigned)p->n_near_pairs, 256, smem, st>>>(d_C, p->d_ijk, p->d_nb, p->d_off, p->d_P,
-                                                                         d_pa, p->d_near_src, p->d_near_boff,
-                                                                         p->n_near_pairs, p->d_Nblk);
+        IE_CK(cudaFuncSetAttribute(near_blocks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)sizeof(SmemNear)));
+        near_blocks_kernel<<<(unsigned)p->n_near_pairs, kNearThreads, sizeof(SmemNear), st>>>(
+            d_C, p->d_ijk, p->d_nb, p->d_off, p->d_P, d_pa, p->d_near_src, p->d_near_boff, p->d_Nblk, p->d_Nshort);
     }
     IE_CK_LAUNCH();
     IE_CK(cudaFreeAsync(d_ds, st));

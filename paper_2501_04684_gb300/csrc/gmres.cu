@@ -896,9 +896,9 @@ ie_status ie_solver_create(ie_plan p, int nrhs, const ie_solve_opts *opts, ie_so
         set_error("solver set-up copies failed");
         return fail(IE_ERR_CUDA);
     }
-    // work lists must exist before graph capture (they allocate)
+    // work lists must exist before graph capture (they allocate); the convolution has none
     WorkList *wl = nullptr;
-    e = work_list_for(p, o.prec, R, &wl);
+    e = conv_full(p, o.prec) ? IE_OK : work_list_for(p, o.prec, R, &wl);
     if (e != IE_OK) return fail(e);
     if (cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&s->ev, cudaEventDisableTiming) != cudaSuccess) {

@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <array>
 #include <atomic>
 #include <map>
 #include <mutex>
@@ -134,6 +135,24 @@ struct WorkList {
     int64_t n = 0;
 };
 
+// The far product as a lattice convolution (conv.cu): scatterers of one padded size.
+constexpr int kNearReach = 4;        // site pairs of adjacent boxes beyond this many lattice steps are convolved
+constexpr unsigned kConvMask =
+    IE_PRECMASK(IE_PREC_FP32) | IE_PRECMASK(IE_PREC_BF16X3) | IE_PRECMASK(IE_PREC_FP16X3);
+struct ConvUse {
+    unsigned full = 0, far = 0;                  // precisions of IE_FULL products, of far products and translations
+};
+struct ConvClass {
+    int L[3] = {0, 0, 0}, E[3] = {0, 0, 0};      // transform lengths, largest box extents
+    std::vector<int32_t> group;                  // scatterers
+    std::vector<std::array<int32_t, 3>> lo;      // their lowest boxes
+    int64_t a_col = 0, b_col = 0;                // workspace elements of one column
+    int chunk = 1;                               // columns in flight
+    int32_t *d_slot = nullptr, *d_cols = nullptr;
+    float2 *d_tw = nullptr;
+    float4 *d_K = nullptr;
+};
+
 }  // namespace ie
 
 // A coupling-block store shared by plans (ie_store_create): the canonical far blocks of
@@ -220,6 +239,22 @@ struct ie_plan_s {
     int64_t *d_near_boff = nullptr;    // n_near_pairs (element offset into d_Nblk)
     float2 *d_Nblk = nullptr;          // blocks, nb_a x nb_b column-major each
 
+    // far product as a lattice convolution (empty: block products only)
+    std::vector<ie::ConvClass> conv;
+    ie::ConvUse conv_use;              // products that take it
+    float2 *d_convA = nullptr, *d_convB = nullptr;
+    int32_t *d_box_cols = nullptr;     // [nbox] right-hand sides of each box's scatterer (null: all)
+    float2 *d_Nshort = nullptr;        // near blocks of the site pairs within kNearReach (as d_Nblk)
+    // adjacent pairs (26 groups) whose site pairs beyond kNearReach the convolution holds,
+    // with the negated blocks of just those site pairs
+    int64_t n_adj = 0;
+    std::vector<int64_t> h_adj_start;  // 28 (groups e = (ex+1)*9 + (ey+1)*3 + (ez+1))
+    std::vector<int32_t> h_adj_src;    // kept only with gnrhs
+    int32_t *d_adj_src = nullptr, *d_adj_dst = nullptr;
+    float2 *d_Cadj = nullptr;          // [27][192 (k)][192 (m)]
+    uint16_t *d_Cadj_bf16 = nullptr, *d_Cadj_fp16 = nullptr;
+    int32_t *d_Cadj_exp16 = nullptr;
+
     // scratch (sized for max_rhs)
     float2 *d_X = nullptr;             // [max_rhs][nbox][192]
     float2 *d_Yslab = nullptr;         // [kSlabs][max_rhs][nbox][192]
@@ -230,6 +265,7 @@ struct ie_plan_s {
     float2 *d_tmp = nullptr;           // [max_rhs][n] scratch of products
 
     std::map<int, ie::WorkList> simt_work, tc_work;   // keyed by nrhs (tensor core: and its tuning)
+    std::map<int, ie::WorkList> adj_work;             // adjacent pairs, keyed by 2 nrhs + tensor core
     std::map<int, std::pair<int, int>> tc_tuned;      // nrhs -> (tile columns, item order) from ie_plan_tune
     std::vector<void *> allocs;
     size_t bytes = 0;
@@ -262,12 +298,29 @@ ie_status launch_coupling_simt(const ie_plan p, const int32_t *d_disp, int64_t n
 // 16-bit split images (and, fp16, the per-block exponents) of nd FP32 blocks [k][m].
 ie_status launch_coupling_tc(const float2 *Cs, int64_t nd, uint16_t *out, int32_t *exps, bool fp16, cudaStream_t st);
 ie_status launch_near_blocks(ie_plan p, cudaStream_t st);
+
+// ---- far product as a lattice convolution (conv.cu)
+// the classes of a problem's scatterers (nblocks: stored blocks its pairs use) and what they serve
+ConvUse conv_classes(const ie_problem *pr, int64_t npairs, int64_t nblocks, std::vector<ConvClass> &out);
+size_t conv_bytes(const ie_problem *pr, const std::vector<ConvClass> &cl, const ConvUse &use, int64_t nadj,
+                  int64_t near_elems);
+int64_t conv_traffic(const ie_plan_s *p, int nrhs);
+ie_status conv_create(ie_plan p, cudaStream_t st);
+// Y = K' * X at every box (zero in columns a scatterer does not have)
+ie_status launch_conv(ie_plan p, const float2 *X, float2 *Y, int nrhs, cudaStream_t st, const int *gate);
+inline bool conv_full(const ie_plan_s *p, int prec) { return (p->conv_use.full & IE_PRECMASK(prec)) != 0; }
+inline bool conv_far(const ie_plan_s *p, int prec) { return (p->conv_use.far & IE_PRECMASK(prec)) != 0; }
+// Slab += the (negated) product of the adjacent pairs' convolved site pairs
+ie_status launch_adjacent(ie_plan p, int prec, const float2 *X, float2 *slab, int nrhs, cudaStream_t st,
+                          const int *gate);
+ie_status adj_list(ie_plan p, bool tc, int nrhs, WorkList **out);
 ie_status launch_aggregate(const ie_plan p, const float2 *c, float2 *X, int nrhs, cudaStream_t st,
                            const int *gate = nullptr);
 // symmetry = 1: the 48 signed-permuted FP32 copies of X into p->d_Xsym
 ie_status launch_permute_sym(const ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate = nullptr);
+// plain: without the symmetric store's permuted copies
 ie_status launch_split_tc(const ie_plan p, const float2 *X, int nrhs, bool fp16, cudaStream_t st,
-                          const int *gate = nullptr);
+                          const int *gate = nullptr, bool plain = false);
 ie_status launch_disaggregate(const ie_plan p, const float2 *Yslab, int nslab, size_t slab_stride, float2 *r,
                               int nrhs, bool accumulate, cudaStream_t st, const int *gate = nullptr);
 ie_status launch_sum_slabs(const ie_plan p, const float2 *Yslab, int nslab, size_t slab_stride, float2 *Y, int nrhs,
@@ -276,10 +329,11 @@ ie_status launch_zero(void *ptr, size_t bytes, cudaStream_t st, const int *gate 
 // nslab regions of `count` complex values, `stride` complex values apart, in one launch
 ie_status launch_zero_slabs(float2 *base, int nslab, size_t stride, size_t count, cudaStream_t st,
                             const int *gate = nullptr);
+// shorter: only the site pairs within kNearReach (the others are in the convolution)
 ie_status launch_near(const ie_plan p, const float2 *c, float2 *y, int nrhs, cudaStream_t st,
-                      const int *gate = nullptr);
+                      const int *gate = nullptr, bool shorter = false);
 ie_status launch_translate_simt(ie_plan p, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
-                                const int *gate = nullptr);
+                                const int *gate = nullptr, bool adjacent = false);
 ie_status launch_translate_cvfcnn(ie_plan p, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
                                   const int *gate = nullptr);
 // fits the surrogates of the ncanon canonical displacements (device, ncanon x 3); with
@@ -288,8 +342,9 @@ ie_status launch_translate_cvfcnn(ie_plan p, const float2 *X, float2 *Yslab, int
 // network turned into its own frame, else the canonical networks are the stored blocks'
 ie_status launch_cvfcnn_fit(ie_plan p, const int32_t *canon_disp, int64_t ncanon, const int32_t *gcanon,
                             const int32_t *gsigma, const uint16_t *map, cudaStream_t st);
+// adjacent: the adjacent pairs' blocks instead of the far ones (one slab)
 ie_status launch_translate_tc(ie_plan p, int prec, float2 *Yslab, int nrhs, cudaStream_t st,
-                              const int *gate = nullptr);
+                              const int *gate = nullptr, bool adjacent = false);
 ie_status launch_plane_wave(const ie_plan p, const double *d_khat, const double *d_pol, int nrhs, float2 *v,
                             cudaStream_t st);
 
@@ -303,8 +358,10 @@ ie_status work_list(ie_plan p, bool tc, int nrhs, WorkList **out, int max_cols =
 // The work list the translation of precision `prec` launches with (the same cache entry):
 // made ahead of a stream capture, since building one allocates.
 ie_status work_list_for(ie_plan p, int prec, int nrhs, WorkList **out);
+// part: every site pair, those within kNearReach lattice steps, or the others negated
+enum BlockPart { kAllSites = 0, kShortSites = 1, kLongSitesNegated = 2 };
 ie_status launch_coupling_fp32(double k, double eta, double a, const int32_t *d_disp, int64_t nd, float2 *out,
-                               bool row_major, cudaStream_t st);
+                               bool row_major, cudaStream_t st, BlockPart part = kAllSites);
 // FP32 blocks of nd displacements (kept in C32 when given, else cut chunk by chunk from a
 // staging buffer) and their 16-bit images where the buffers are given
 ie_status generate_blocks(double k, double eta, double a, const int32_t *d_disp, int64_t nd, float2 *C32,

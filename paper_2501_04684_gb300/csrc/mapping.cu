@@ -274,9 +274,11 @@ ie_status launch_aggregate(const ie_plan p, const float2 *c, float2 *X, int nrhs
     return IE_OK;
 }
 
-ie_status launch_split_tc(const ie_plan p, const float2 *X, int nrhs, bool fp16, cudaStream_t st, const int *gate) {
-    const dim3 grid(p->nbox, nrhs, p->sym ? kSym : 1);
-    const uint16_t *map = p->sym ? p->d_symmap : nullptr;
+ie_status launch_split_tc(const ie_plan p, const float2 *X, int nrhs, bool fp16, cudaStream_t st, const int *gate,
+                          bool plain) {
+    const bool sym = p->sym && !plain;
+    const dim3 grid(p->nbox, nrhs, sym ? kSym : 1);
+    const uint16_t *map = sym ? p->d_symmap : nullptr;
     if (fp16)
         split_kernel<true><<<grid, kNU, 0, st>>>(X, p->nbox, nrhs, p->d_Xtc, p->d_Xexp, p->d_Xinf, map, gate);
     else

@@ -20,8 +20,8 @@ template <int ROWS>
 __global__ void __launch_bounds__(kNearWarps * 32, 2)
 near_kernel(const int32_t *__restrict__ nb, const int64_t *__restrict__ off, int64_t n,
             const int32_t *__restrict__ start, const int32_t *__restrict__ src,
-            const int64_t *__restrict__ boff, const float2 *__restrict__ Nblk,
-            const double *__restrict__ alpha_box,
+            const int64_t *__restrict__ boff, const float2 *__restrict__ Nblk, const float2 *__restrict__ Nbeyond,
+            const int32_t *__restrict__ box_cols, const double *__restrict__ alpha_box,
             const float2 *__restrict__ c, float2 *__restrict__ y, const int *__restrict__ gate) {
     if (gate && *gate == 0) return;
     constexpr int G = ROWS == 1 ? 16 : (ROWS == 2 ? 8 : 4);     // columns per load group
@@ -31,6 +31,7 @@ near_kernel(const int32_t *__restrict__ nb, const int64_t *__restrict__ off, int
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int na = nb[a];
     const float2 *cr = c + (int64_t)r * n;
+    if (box_cols && r >= box_cols[a]) Nblk = Nbeyond;   // a column without far part: every site pair
     double2 acc[ROWS];
 #pragma unroll
     for (int k = 0; k < ROWS; ++k) acc[k] = make_double2(0, 0);
@@ -98,19 +99,24 @@ near_kernel(const int32_t *__restrict__ nb, const int64_t *__restrict__ off, int
 
 }  // namespace
 
-ie_status launch_near(const ie_plan p, const float2 *c, float2 *y, int nrhs, cudaStream_t st, const int *gate) {
+ie_status launch_near(const ie_plan p, const float2 *c, float2 *y, int nrhs, cudaStream_t st, const int *gate,
+                      bool shorter) {
+    const float2 *blocks = shorter ? p->d_Nshort : p->d_Nblk;
     int maxnb = 0;
     for (int v : p->nb) maxnb = v > maxnb ? v : maxnb;
     const dim3 grid(p->nbox, nrhs);
     if (maxnb <= 32)
         near_kernel<1><<<grid, kNearWarps * 32, 0, st>>>(p->d_nb, p->d_off, p->n, p->d_near_start, p->d_near_src,
-                                                         p->d_near_boff, p->d_Nblk, p->d_alpha_box, c, y, gate);
+                                                         p->d_near_boff, blocks, p->d_Nblk,
+                                                         shorter ? p->d_box_cols : nullptr, p->d_alpha_box, c, y, gate);
     else if (maxnb <= 64)
         near_kernel<2><<<grid, kNearWarps * 32, 0, st>>>(p->d_nb, p->d_off, p->n, p->d_near_start, p->d_near_src,
-                                                         p->d_near_boff, p->d_Nblk, p->d_alpha_box, c, y, gate);
+                                                         p->d_near_boff, blocks, p->d_Nblk,
+                                                         shorter ? p->d_box_cols : nullptr, p->d_alpha_box, c, y, gate);
     else
         near_kernel<6><<<grid, kNearWarps * 32, 0, st>>>(p->d_nb, p->d_off, p->n, p->d_near_start, p->d_near_src,
-                                                         p->d_near_boff, p->d_Nblk, p->d_alpha_box, c, y, gate);
+                                                         p->d_near_boff, blocks, p->d_Nblk,
+                                                         shorter ? p->d_box_cols : nullptr, p->d_alpha_box, c, y, gate);
     IE_CK_LAUNCH();
     return IE_OK;
 }

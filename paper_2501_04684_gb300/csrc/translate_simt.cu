@@ -193,8 +193,16 @@ ie_status prepare_translate_simt() {
 }
 
 ie_status launch_translate_simt(ie_plan p, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
-                                const int *gate) {
+                                const int *gate, bool adjacent) {
     WorkList *wl = nullptr;
+    if (adjacent) {     // one block per displacement, at most 26 terms per target: one slab
+        IE_TRY(adj_list(p, false, nrhs, &wl));
+        if (wl->n == 0) return IE_OK;
+        translate_simt_kernel<<<(unsigned)wl->n, kThreads, sizeof(SmemSimt), st>>>(
+            wl->d_items, p->d_Cadj, p->d_adj_src, p->d_adj_dst, X, Yslab, 0, p->nbox, nrhs, SymArgs(), gate);
+        IE_CK_LAUNCH();
+        return IE_OK;
+    }
     IE_TRY(work_list_for(p, IE_PREC_FP32, nrhs, &wl));
     if (wl->n == 0) return IE_OK;
     if (!p->d_Csimt) return set_error("the plan holds no FP32 coupling store"), IE_ERR_UNSUPPORTED;

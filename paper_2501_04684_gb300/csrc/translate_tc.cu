@@ -682,45 +682,47 @@ ie_status prepare_translate_tc() {
     return IE_OK;
 }
 
-ie_status launch_translate_tc(ie_plan p, int prec, float2 *Yslab, int nrhs, cudaStream_t st, const int *gate) {
+ie_status launch_translate_tc(ie_plan p, int prec, float2 *Yslab, int nrhs, cudaStream_t st, const int *gate,
+                              bool adjacent) {
     const bool fp16 = is_fp16(prec);
-    const uint16_t *C = fp16 ? p->d_Cfp16 : p->d_Cbf16;
+    const uint16_t *C = adjacent ? (fp16 ? p->d_Cadj_fp16 : p->d_Cadj_bf16) : (fp16 ? p->d_Cfp16 : p->d_Cbf16);
     if (!C) return set_error("tensor-core coupling store for precision %d not built", prec), IE_ERR_UNSUPPORTED;
     if ((int64_t)p->max_rhs * p->nbox * kNU > (int64_t)INT32_MAX)
         return set_error("plan too large for the tensor-core translation's 32-bit offsets"), IE_ERR_UNSUPPORTED;
     WorkList *wl = nullptr;
-    IE_TRY(work_list_for(p, prec, nrhs, &wl));
+    IE_TRY(adjacent ? adj_list(p, true, nrhs, &wl) : work_list_for(p, prec, nrhs, &wl));
     if (wl->n == 0) return IE_OK;
+    const bool sym = p->sym && !adjacent;       // the adjacent pairs have a block per displacement
     TcArgs a;
     a.items = wl->d_items;
     a.n_items = wl->n;
     a.C = C;
-    a.Cexp = fp16 ? p->d_Cexp16 : nullptr;
+    a.Cexp = !fp16 ? nullptr : adjacent ? p->d_Cadj_exp16 : p->d_Cexp16;
     a.Xexp = p->d_Xexp;
     a.Xtc = p->d_Xtc;
     a.plane = (int64_t)nrhs * p->nbox * 2 * kNU;
-    a.src = p->d_src;
-    a.dst = p->d_dst;
+    a.src = adjacent ? p->d_adj_src : p->d_src;
+    a.dst = adjacent ? p->d_adj_dst : p->d_dst;
     a.Yslab = reinterpret_cast<float *>(Yslab);
-    a.slab_stride = slab_stride(p);
+    a.slab_stride = adjacent ? 0 : slab_stride(p);   // at most 26 terms per target: one slab
     a.nbox = p->nbox;
     a.nrhs = nrhs;
     a.err = p->d_err;
     a.gate = gate;
-    a.gcanon = p->sym ? p->d_gcanon : nullptr;
-    a.gsigma = p->sym ? p->d_gsigma : nullptr;
-    a.symmap = p->sym ? p->d_symmap : nullptr;
+    a.gcanon = sym ? p->d_gcanon : nullptr;
+    a.gsigma = sym ? p->d_gsigma : nullptr;
+    a.symmap = sym ? p->d_symmap : nullptr;
     a.sig_stride = 2 * a.plane;
-    a.pgroup = p->sym ? p->d_pgroup : nullptr;   // the symmetric store's items are packed
+    a.pgroup = sym ? p->d_pgroup : nullptr;   // the symmetric store's items are packed
     int grid = (int)std::min<int64_t>(wl->n, (int64_t)kCtasPerSm * (p->tc_sms > 0 ? p->tc_sms : 148));
     if (prec == IE_PREC_BF16X3)
-        launch_tc<false, true>(a, grid, p->sym, st);
+        launch_tc<false, true>(a, grid, sym, st);
     else if (prec == IE_PREC_FP16X3)
-        launch_tc<true, true>(a, grid, p->sym, st);
+        launch_tc<true, true>(a, grid, sym, st);
     else if (prec == IE_PREC_BF16X1)
-        launch_tc<false, false>(a, grid, p->sym, st);
+        launch_tc<false, false>(a, grid, sym, st);
     else if (prec == IE_PREC_FP16X1)
-        launch_tc<true, false>(a, grid, p->sym, st);
+        launch_tc<true, false>(a, grid, sym, st);
     else
         return set_error("not a tensor-core precision: %d", prec), IE_ERR_INVALID;
     IE_CK_LAUNCH();

@@ -6,7 +6,9 @@ Example (the translation kernel of one BF16X3 product):
 
   python -m paper_2501_04684_gb300.profile_case --grid 10 --radius 4 --prec bf16x3
 
-With --prec cvfcnn the plan fits the translation networks (FP64 Jacobi SVDs); --map N also
+At the default box edge lambda/4 the fp32, bf16x3 and fp16x3 products are lattice convolutions
+(kernels conv_*); --edge 256 (box edge lambda/256) profiles their block-product kernels on the
+same geometry.  With --prec cvfcnn the plan fits the translation networks (FP64 Jacobi SVDs); --map N also
 runs the mapping construction for N boxes' worth of seeded point-dipole functions.
 """
 from __future__ import annotations
@@ -26,6 +28,8 @@ def main():
     ap.add_argument("--reps", type=int, default=2)
     ap.add_argument("--nrhs", type=int, default=1)
     ap.add_argument("--symmetry", type=int, default=0, choices=[0, 1])
+    ap.add_argument("--edge", type=float, default=4.0, help="box edge lambda / EDGE")
+    ap.add_argument("--which", default="far", choices=["far", "full"])
     ap.add_argument("--map", type=int, default=0,
                     help="also map this many boxes' worth of seeded point-dipole functions (ie_map_basis)")
     args = ap.parse_args()
@@ -39,6 +43,8 @@ def main():
     precs = [names[s] for s in args.prec.split(",")]
     boxes = W.sphere_shell(args.grid, args.radius)
     p = W.make_problem("profile", args.grid, boxes, 32, seed_P=61, alpha=1.0)
+    p.a = 1.0 / args.edge
+    which = {"far": ie.IE_FAR, "full": ie.IE_FULL}[args.which]
     mask = ie.precmask(*precs)
     with ie.Plan(ie.problem_from(p, mask, args.nrhs, symmetry=args.symmetry)) as plan:
         st = plan.stats
@@ -46,7 +52,7 @@ def main():
         y = torch.zeros_like(c)
         for prec in precs:
             for _ in range(args.reps):
-                ie.ie_matvec(plan.handle, ie.IE_FAR, prec, c, y, args.nrhs)
+                ie.ie_matvec(plan.handle, which, prec, c, y, args.nrhs)
         torch.cuda.synchronize()
         if args.map:
             fun_off, pos, mom = W.point_dipole_basis(p.nb[:args.map], 63, a=p.a)
