@@ -3,9 +3,9 @@
 // (3 N_s x 192) at N_s Fibonacci samples on a sphere S about the box centre; a
 // function radiates B_f there (eq. 4); eq. 11 takes C_f = A^+ B_f, row f of P_b.
 //
-// A is the same for every box, so A^+ is formed once: a Householder QR of A in one
-// CTA, then one warp per unit vector e_i applies Q^H and back-substitutes with R,
-// which gives column i of A^+ = R^-1 Q_1^H.  With a Tikhonov weight the factorised
+// A is the same for every box, so A^+ is formed once: a Householder QR of A by one CTA per
+// column with the columns of Q_1 formed from the reflectors, then one warp per sample row
+// back-substitutes with R, which gives column i of A^+ = R^-1 Q_1^H.  With a Tikhonov weight the factorised
 // matrix is [A; lambda I] (lambda = t ||A||_F) and the first 3 N_s columns of its
 // pseudo-inverse are (A^H A + lambda^2 I)^-1 A^H.  The per-function work (fields on S,
 // the product with A^+, the residual on S) is one CTA per 8 functions.  All FP64:
@@ -22,8 +22,7 @@ namespace {
 constexpr int kMinSamples = 64;                   // 3 N_s >= 192: full column rank possible
 constexpr int kMaxSamples = 256;
 constexpr int kFunPerCta = 8;
-constexpr int kMapThreads = 256;
-constexpr int kPinvWarps = 8;
+constexpr int kMapThreads = 2 * kNU;
 constexpr int64_t kMapChunk = int64_t(1) << 16;   // functions per device pass
 
 struct Sphere {
@@ -31,20 +30,10 @@ struct Sphere {
     int ns;                     // samples on S
 };
 
-__device__ inline double2 cmul(double2 a, double2 b) {
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+__device__ inline void cmac(double2 &acc, double2 a, double2 b) {   // acc += a b
+    acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
+    acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
 }
-__device__ inline double2 cmul_conj(double2 a, double2 b) {   // conj(a) * b
-    return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
-}
-__device__ inline double2 warp_sum2(double2 v) {
-    for (int o = 16; o; o >>= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-    }
-    return v;
-}
-
 // Sample l of the spherical Fibonacci lattice on S: polar angle arccos(1 - (2l+1)/N_s),
 // azimuth 2 pi l / golden ratio.
 __device__ inline void sample_point(const Sphere &s, int l, double r[3]) {
@@ -85,130 +74,200 @@ __global__ void sample_matrix_kernel(Sphere s, double2 *__restrict__ A, int lda,
         }
 }
 
-// Householder QR of A (m x 192, column-major) in one CTA.  Step j maps column j below
-// the diagonal onto alpha e_j with H_j = I - tau_j v_j v_j^H, alpha = -e^{i arg x0} ||x||,
-// v_j = x - alpha e_j (stored in V, rows j..m-1), tau_j = 2 / ||v_j||^2; R stays in the
-// upper triangle of A.  *status = 1 if a column is zero (rank deficient).
-// tikhonov > 0: rows m_data .. m_data+191 (zero on entry) first receive lambda I,
-// lambda = tikhonov * ||A[0 .. m_data)||_F.
-__global__ void __launch_bounds__(1024) householder_qr_kernel(double2 *__restrict__ A, int m, int m_data,
-                                                              double tikhonov, double2 *__restrict__ V,
-                                                              double *__restrict__ tau, int *__restrict__ status) {
-    __shared__ double red[32];
-    __shared__ double2 s_v0;
-    __shared__ double s_tau;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
-    if (tikhonov > 0.0) {
-        double ss = 0.0;
-        for (int c = 0; c < kNU; ++c)
-            for (int i = tid; i < m_data; i += blockDim.x) {
-                const double2 x = A[i + (size_t)m * c];
-                ss += x.x * x.x + x.y * x.y;
-            }
-        for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (lane == 0) red[warp] = ss;
-        __syncthreads();
-        if (tid < kNU) {
-            double tot = 0.0;
-            for (int w = 0; w < nwarp; ++w) tot += red[w];
-            A[(m_data + tid) + (size_t)m * tid] = make_double2(tikhonov * sqrt(tot), 0.0);
+// Pseudo-inverse, first part: the Householder QR of A (m x 192, column-major, m <= 960), one
+// CTA per column, the columns in registers.  Step j maps column j below the diagonal onto
+// alpha e_j with H_j = I - tau_j v_j v_j^H, alpha = -e^{i arg x0} ||x||, v_j = x - alpha e_j
+// (V, rows j..m-1), tau_j = 2 / ||v_j||^2; R goes to the upper triangle of A.  CTA j publishes
+// v_j and raises flag[j]; the later CTAs apply it, CTA j + 1 then publishes at once.  Then
+// each CTA forms its column of Q_1 = H_0 .. H_191 [I; 0] (conjugated rows, Y[i][c], i <
+// m_data), needing only the published vectors.  *status = 1 if a column is zero (rank
+// deficient), 2 if a wait gave up.
+// tikhonov > 0: rows m_data .. m_data+191 are lambda I, lambda = tikhonov ||A[0 .. m_data)||_F.
+// Bound by the chain of 192 steps, and a step by FP64 issue (64 cycles per warp instruction and
+// SM quarter): four warps per CTA, one per quarter, no row outside [j, m), re and im reduced
+// in one shuffle tree.  m = 576: 2.5 ms; all columns in one CTA took 37 ms.
+constexpr int kQrThreads = 128, kQrWarps = kQrThreads / 32, kQrRows = 8;
+static_assert(kQrRows * kQrThreads >= 3 * kMaxSamples + kNU, "columns in registers");
+constexpr long long kQrWaitCycles = 1ll << 31;      // bounded wait, ~1 s
+
+// Sum over the block, the result in every thread.  The first exchange leaves re in the lower
+// and im in the upper half-warp.
+__device__ inline double2 block_sum(double2 v, double (*red)[2][kQrWarps], int &slot) {
+    const int lane = threadIdx.x & 31, hi = lane >> 4;
+    double x = (hi ? v.y : v.x) + __shfl_xor_sync(0xffffffffu, hi ? v.x : v.y, 16);
+    for (int o = 8; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((lane & 15) == 0) red[slot][hi][threadIdx.x >> 5] = x;
+    __syncthreads();
+    const double *r = red[slot][0], *i = red[slot][1];
+    slot ^= 1;          // two buffers: one barrier per sum
+    return make_double2((r[0] + r[1]) + (r[2] + r[3]), (i[0] + i[1]) + (i[2] + i[3]));
+}
+static_assert(kQrWarps == 4, "four partial sums");
+
+__global__ void __launch_bounds__(kQrThreads) qr_kernel(double2 *__restrict__ A, const double2 *__restrict__ A0, int m,
+                                                        int m_data, double tikhonov, double2 *V, double *tau, int *flag,
+                                                        double2 *__restrict__ Y, int *__restrict__ status) {
+    __shared__ double red[2][2][kQrWarps];
+    __shared__ double2 s_x0, s_ph;
+    __shared__ double s_ax0;
+    __shared__ int s_ok;
+    const int tid = threadIdx.x, c = blockIdx.x, w0 = tid & ~31;
+    int slot = 0;
+    double lambda = 0.0;
+    if (tikhonov > 0.0) {       // every CTA sums ||A||_F itself, in the same order, from the copy
+        double2 ss = make_double2(0.0, 0.0);    // (R already replaces columns of A elsewhere)
+        for (int i = tid; i < m_data * kNU; i += kQrThreads) {
+            const double2 x = A0[i];
+            ss.x = fma(x.x, x.x, ss.x), ss.y = fma(x.y, x.y, ss.y);
         }
-        __syncthreads();
+        ss = block_sum(ss, red, slot);
+        lambda = tikhonov * sqrt(ss.x + ss.y);
     }
-    for (int j = 0; j < kNU; ++j) {
-        double2 *a = A + (size_t)m * j;
-        double ss = 0.0;
-        for (int i = j + tid; i < m; i += blockDim.x) ss += a[i].x * a[i].x + a[i].y * a[i].y;
-        for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (lane == 0) red[warp] = ss;
-        __syncthreads();
+    double2 x[kQrRows];
+#pragma unroll
+    for (int t = 0; t < kQrRows; ++t) {
+        const int i = tid + t * kQrThreads;
+        x[t] = i < m_data ? A[i + (size_t)m * c] : make_double2(i < m && i - m_data == c ? lambda : 0.0, 0.0);
+    }
+    // rows of this warp's chunk t that a step over rows [j, m) touches
+    auto live = [&](int t, int j) { return w0 + t * kQrThreads < m && w0 + t * kQrThreads + 31 >= j; };
+    double2 v[kQrRows];
+    auto fetch = [&](int j) {
+#pragma unroll
+        for (int t = 0; t < kQrRows; ++t) {
+            const int i = tid + t * kQrThreads;
+            v[t] = live(t, j) && i < m ? __ldcg(V + i + (size_t)m * j) : make_double2(0.0, 0.0);
+        }
+    };
+    // x <- H_j x, v = v_j (zero above row j)
+    auto reflect = [&](int j, double tj) {
+        double2 d = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int t = 0; t < kQrRows; ++t)
+            if (live(t, j)) {
+                d.x = fma(v[t].x, x[t].x, fma(v[t].y, x[t].y, d.x));
+                d.y = fma(v[t].x, x[t].y, fma(-v[t].y, x[t].x, d.y));
+            }
+        d = block_sum(d, red, slot);
+        const double fx = tj * d.x, fy = tj * d.y;
+#pragma unroll
+        for (int t = 0; t < kQrRows; ++t)
+            if (live(t, j)) {
+                x[t].x = fma(-fx, v[t].x, fma(fy, v[t].y, x[t].x));
+                x[t].y = fma(-fx, v[t].y, fma(-fy, v[t].x, x[t].y));
+            }
+    };
+    for (int j = 0; j < c; ++j) {
         if (tid == 0) {
-            double tot = 0.0;
-            for (int w = 0; w < nwarp; ++w) tot += red[w];
-            double xn = sqrt(tot);
-            double2 x0 = a[j];
-            double ax0 = hypot(x0.x, x0.y);
-            double2 ph = ax0 > 0.0 ? make_double2(x0.x / ax0, x0.y / ax0) : make_double2(1.0, 0.0);
-            if (xn == 0.0) {
-                *status = 1;
-                s_tau = 0.0;
-                s_v0 = make_double2(0.0, 0.0);
-            } else {
-                s_v0 = make_double2(ph.x * (ax0 + xn), ph.y * (ax0 + xn));
-                s_tau = 1.0 / (xn * (xn + ax0));            // ||v||^2 = 2 xn (xn + |x0|)
-                a[j] = make_double2(-ph.x * xn, -ph.y * xn);  // R_jj = alpha
-            }
-            tau[j] = s_tau;
+            const long long t0 = clock64();
+            int f = 0;
+            while (!f && clock64() - t0 < kQrWaitCycles)
+                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(f) : "l"(flag + j) : "memory");
+            s_ok = f;
         }
         __syncthreads();
-        double2 *v = V + (size_t)m * j;
-        for (int i = j + tid; i < m; i += blockDim.x) v[i] = (i == j) ? s_v0 : a[i];
-        __syncthreads();
-        for (int c = j + 1 + warp; c < kNU; c += nwarp) {
-            double2 *ac = A + (size_t)m * c;
-            double2 d = make_double2(0.0, 0.0);
-            for (int i = j + lane; i < m; i += 32) {
-                double2 t = cmul_conj(v[i], ac[i]);
-                d.x += t.x;
-                d.y += t.y;
-            }
-            d = warp_sum2(d);
-            double2 f = make_double2(s_tau * d.x, s_tau * d.y);
-            for (int i = j + lane; i < m; i += 32) {
-                double2 t = cmul(f, v[i]);
-                ac[i].x -= t.x;
-                ac[i].y -= t.y;
-            }
+        if (!s_ok) {            // the same in every thread
+            if (tid == 0) atomicMax(status, 2);
+            return;
+        }
+        fetch(j);
+        reflect(j, __ldcg(tau + j));
+    }
+    double tc;
+    {   // the reflector of the own column
+        double2 ss = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int t = 0; t < kQrRows; ++t) {
+            const int i = tid + t * kQrThreads;
+            if (i == c) s_x0 = x[t];
+            if (live(t, c) && i >= c) ss.x = fma(x[t].x, x[t].x, ss.x), ss.y = fma(x[t].y, x[t].y, ss.y);
         }
         __syncthreads();
+        const double2 x0 = s_x0;
+        if (w0 == 32 * (kQrWarps - 1)) {       // beside the other warps' sums
+            const double ax = hypot(x0.x, x0.y);
+            if (tid == w0) {
+                s_ax0 = ax;
+                s_ph = ax > 0.0 ? make_double2(x0.x / ax, x0.y / ax) : make_double2(1.0, 0.0);
+            }
+        }
+        ss = block_sum(ss, red, slot);
+        const double xn = sqrt(ss.x + ss.y), ax0 = s_ax0;
+        const double2 ph = s_ph;
+        tc = xn > 0.0 ? 1.0 / (xn * (xn + ax0)) : 0.0;             // ||v||^2 = 2 xn (xn + |x0|)
+#pragma unroll
+        for (int t = 0; t < kQrRows; ++t) {
+            const int i = tid + t * kQrThreads;
+            v[t] = i > c ? x[t] : make_double2(0.0, 0.0);
+            if (i == c && xn > 0.0) v[t] = make_double2(ph.x * (ax0 + xn), ph.y * (ax0 + xn));
+            if (i < m) V[i + (size_t)m * c] = v[t];
+            if (i <= c)         // column c of R, R_cc = alpha
+                A[i + (size_t)m * c] = i < c ? x[t] : make_double2(-ph.x * xn, -ph.y * xn);
+        }
+        if (tid == 0) {
+            tau[c] = tc;
+            if (xn == 0.0) atomicMax(status, 1);
+        }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(flag + c) : "memory");
+    }
+    // column c of Q_1: H_c .. H_0 applied to e_c (H_j with j > c leaves it as it is)
+#pragma unroll
+    for (int t = 0; t < kQrRows; ++t) x[t] = make_double2(tid + t * kQrThreads == c ? 1.0 : 0.0, 0.0);
+    reflect(c, tc);
+    for (int j = c - 1; j >= 0; --j) {
+        fetch(j);
+        reflect(j, __ldcg(tau + j));
+    }
+#pragma unroll
+    for (int t = 0; t < kQrRows; ++t) {
+        const int i = tid + t * kQrThreads;
+        if (i < m_data) Y[(size_t)i * kNU + c] = make_double2(x[t].x, -x[t].y);
     }
 }
 
-// Column i < m_out of the pseudo-inverse of the factorised m-row matrix (stored as row i
-// of Apinv, [m_out][192]): y = Q^H e_i = H_191 ... H_0 e_i, then R x = y[0..192) by back
-// substitution.  One warp per i, y in shared memory.
-__global__ void pinv_kernel(const double2 *__restrict__ R, const double2 *__restrict__ V,
-                            const double *__restrict__ tau, int m, int m_out, double2 *__restrict__ Apinv) {
-    extern __shared__ double2 ys[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * kPinvWarps + warp;
-    if (i >= m_out) return;   // the whole warp leaves; nothing below synchronises the block
-    double2 *y = ys + (size_t)warp * m;
-    for (int r = lane; r < m; r += 32) y[r] = make_double2(r == i ? 1.0 : 0.0, 0.0);
-    __syncwarp();
-    for (int j = 0; j < kNU; ++j) {
-        const double2 *v = V + (size_t)m * j;
-        double2 d = make_double2(0.0, 0.0);
-        for (int r = j + lane; r < m; r += 32) {
-            double2 t = cmul_conj(v[r], y[r]);
-            d.x += t.x;
-            d.y += t.y;
+// Second part: column i of A^+ = R^-1 Q_1^H (row i of Apinv, [m_data][192]) from row i of
+// conj(Q_1), in place, by back substitution.  One warp per row, six unknowns per lane; the
+// next column of R is in flight during a step.
+__global__ void __launch_bounds__(32) pinv_solve_kernel(const double2 *__restrict__ R, int m, double2 *__restrict__ Y) {
+    const int lane = threadIdx.x;
+    double2 *row = Y + (size_t)blockIdx.x * kNU;
+    double2 y[kNU / 32], r[kNU / 32];
+#pragma unroll
+    for (int t = 0; t < kNU / 32; ++t) y[t] = row[lane + 32 * t];
+    auto fetch = [&](int c) {
+#pragma unroll
+        for (int t = 0; t < kNU / 32; ++t)
+            r[t] = lane + 32 * t <= c ? R[lane + 32 * t + (size_t)m * c] : make_double2(0.0, 0.0);
+    };
+    fetch(kNU - 1);
+#pragma unroll
+    for (int tc = kNU / 32 - 1; tc >= 0; --tc)
+        for (int lc = 31; lc >= 0; --lc) {
+            const int c = 32 * tc + lc;
+            double2 cur[kNU / 32];
+#pragma unroll
+            for (int t = 0; t < kNU / 32; ++t) cur[t] = r[t];
+            if (c > 0) fetch(c - 1);
+            const double2 yr = make_double2(__shfl_sync(0xffffffffu, y[tc].x, lc), __shfl_sync(0xffffffffu, y[tc].y, lc));
+            const double2 rr = make_double2(__shfl_sync(0xffffffffu, cur[tc].x, lc),
+                                            __shfl_sync(0xffffffffu, cur[tc].y, lc));
+            const double den = rr.x * rr.x + rr.y * rr.y;
+            const double2 x = make_double2((yr.x * rr.x + yr.y * rr.y) / den, (yr.y * rr.x - yr.x * rr.y) / den);
+#pragma unroll
+            for (int t = 0; t <= tc; ++t) {
+                const int i = lane + 32 * t;
+                if (i < c) {
+                    y[t].x = fma(-cur[t].x, x.x, fma(cur[t].y, x.y, y[t].x));
+                    y[t].y = fma(-cur[t].x, x.y, fma(-cur[t].y, x.x, y[t].y));
+                } else if (i == c) {
+                    y[t] = x;
+                }
+            }
         }
-        d = warp_sum2(d);
-        const double tj = tau[j];
-        double2 f = make_double2(tj * d.x, tj * d.y);
-        for (int r = j + lane; r < m; r += 32) {
-            double2 t = cmul(f, v[r]);
-            y[r].x -= t.x;
-            y[r].y -= t.y;
-        }
-        __syncwarp();
-    }
-    for (int r = kNU - 1; r >= 0; --r) {
-        double2 rr = R[r + (size_t)m * r];
-        double2 yr = y[r];
-        double den = rr.x * rr.x + rr.y * rr.y;
-        double2 xr = make_double2((yr.x * rr.x + yr.y * rr.y) / den, (yr.y * rr.x - yr.x * rr.y) / den);
-        __syncwarp();
-        if (lane == 0) y[r] = xr;
-        for (int q = lane; q < r; q += 32) {
-            double2 t = cmul(R[q + (size_t)m * r], xr);
-            y[q].x -= t.x;
-            y[q].y -= t.y;
-        }
-        __syncwarp();
-    }
-    for (int u = lane; u < kNU; u += 32) Apinv[(size_t)i * kNU + u] = y[u];
+#pragma unroll
+    for (int t = 0; t < kNU / 32; ++t) row[lane + 32 * t] = y[t];
 }
 
 struct MapArgs {
@@ -224,7 +283,8 @@ struct MapArgs {
 };
 
 // Eight functions per CTA: their fields on S (eq. 4 summed over the point dipoles),
-// C_f = A^+ B_f (eq. 11), and ||A C_f - B_f|| / ||B_f||.
+// C_f = A^+ B_f (eq. 11), and ||A C_f - B_f|| / ||B_f||.  FP64 rate bound: 192 x 384 x 2 complex
+// multiply-adds per function, four FMAs each.
 __global__ void __launch_bounds__(kMapThreads) map_kernel(MapArgs g) {
     extern __shared__ double2 sm[];
     __shared__ double red[2][kFunPerCta][kMapThreads / 32];
@@ -245,35 +305,29 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapArgs g) {
 #pragma unroll
                 for (int al = 0; al < 3; ++al)
 #pragma unroll
-                    for (int be = 0; be < 3; ++be) {
-                        double2 p = cmul(D[3 * al + be], g.mom[3 * d + be]);
-                        e[al].x += p.x;
-                        e[al].y += p.y;
-                    }
+                    for (int be = 0; be < 3; ++be) cmac(e[al], D[3 * al + be], g.mom[3 * d + be]);
             }
         }
 #pragma unroll
         for (int al = 0; al < 3; ++al) B[t * m + 3 * l + al] = e[al];
     }
     __syncthreads();
-    if (threadIdx.x < kNU) {
-        const int u = threadIdx.x;
-        double2 acc[kFunPerCta];
+    {   // C_f = A^+ B_f: a thread makes one unknown of half the functions
+        constexpr int half = kFunPerCta / 2;
+        const int u = threadIdx.x % kNU, t0 = threadIdx.x / kNU * half;
+        double2 acc[half];
 #pragma unroll
-        for (int t = 0; t < kFunPerCta; ++t) acc[t] = make_double2(0.0, 0.0);
+        for (int t = 0; t < half; ++t) acc[t] = make_double2(0.0, 0.0);
+#pragma unroll 2
         for (int i = 0; i < m; ++i) {
             const double2 w = g.Apinv[(size_t)i * kNU + u];
 #pragma unroll
-            for (int t = 0; t < kFunPerCta; ++t) {
-                double2 p = cmul(w, B[t * m + i]);
-                acc[t].x += p.x;
-                acc[t].y += p.y;
-            }
+            for (int t = 0; t < half; ++t) cmac(acc[t], w, B[(t0 + t) * m + i]);
         }
 #pragma unroll
-        for (int t = 0; t < kFunPerCta; ++t) {
-            C[t * kNU + u] = acc[t];
-            if (f0 + t < g.n_fun) g.P[(f0 + t) * kNU + u] = acc[t];
+        for (int t = 0; t < half; ++t) {
+            C[(t0 + t) * kNU + u] = acc[t];
+            if (f0 + t0 + t < g.n_fun) g.P[(f0 + t0 + t) * kNU + u] = acc[t];
         }
     }
     if (!g.res) return;
@@ -285,14 +339,11 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapArgs g) {
         double2 s[kFunPerCta];
 #pragma unroll
         for (int t = 0; t < kFunPerCta; ++t) s[t] = make_double2(0.0, 0.0);
+#pragma unroll 2
         for (int u = 0; u < kNU; ++u) {
             const double2 a = g.A0[i + (size_t)m * u];
 #pragma unroll
-            for (int t = 0; t < kFunPerCta; ++t) {
-                double2 p = cmul(a, C[t * kNU + u]);
-                s[t].x += p.x;
-                s[t].y += p.y;
-            }
+            for (int t = 0; t < kFunPerCta; ++t) cmac(s[t], a, C[t * kNU + u]);
         }
 #pragma unroll
         for (int t = 0; t < kFunPerCta; ++t) {
@@ -326,24 +377,28 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapArgs g) {
     }
 }
 
-// Device buffers of one ie_map_basis call, freed on every return path.
+// Device buffers of one ie_map_basis call, cut from one allocation (an allocation and its
+// release take about 0.1 ms each), freed on every return path.
 struct Scratch {
-    std::vector<void *> ptrs;
+    char *base = nullptr;
+    size_t used = 0;
     ~Scratch() {
-        for (void *p : ptrs) cudaFree(p);
+        if (base) cudaFree(base);
+    }
+    static size_t round(size_t bytes) { return (bytes + 255) / 256 * 256; }
+    ie_status reserve(size_t bytes) {
+        cudaError_t e = cudaMalloc((void **)&base, bytes);
+        if (e == cudaSuccess) return IE_OK;
+        base = nullptr;
+        cudaGetLastError();
+        set_error("cudaMalloc(%zu bytes): %s", bytes, cudaGetErrorString(e));
+        return e == cudaErrorMemoryAllocation ? IE_ERR_OOM : IE_ERR_CUDA;
     }
     template <class T>
-    ie_status get(T **out, size_t count) {
-        *out = nullptr;
-        if (count == 0) return IE_OK;
-        cudaError_t e = cudaMalloc((void **)out, count * sizeof(T));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            set_error("cudaMalloc(%zu bytes): %s", count * sizeof(T), cudaGetErrorString(e));
-            return e == cudaErrorMemoryAllocation ? IE_ERR_OOM : IE_ERR_CUDA;
-        }
-        ptrs.push_back(*out);
-        return IE_OK;
+    T *get(size_t count) {
+        T *p = reinterpret_cast<T *>(base + used);
+        used += round(count * sizeof(T));
+        return p;
     }
 };
 
@@ -401,49 +456,54 @@ extern "C" ie_status ie_map_basis(const ie_mapping_spec *spec, int64_t n_fun, co
     const Sphere s{spec->k, spec->eta, spec->box_edge, spec->sample_radius * spec->box_edge, spec->n_samples};
     const int m = 3 * s.ns;                                      // rows of A
     const int mf = spec->tikhonov > 0.0 ? m + kNU : m;           // rows of the factorised matrix
-    Scratch sc;
-    double2 *A, *A0, *V, *Apinv;
-    double *tau;
-    int *status;
-    IE_TRY(sc.get(&A, (size_t)mf * kNU));
-    IE_TRY(sc.get(&A0, (size_t)m * kNU));
-    IE_TRY(sc.get(&V, (size_t)mf * kNU));
-    IE_TRY(sc.get(&Apinv, (size_t)m * kNU));
-    IE_TRY(sc.get(&tau, kNU));
-    IE_TRY(sc.get(&status, 1));
-    IE_CK(cudaMemsetAsync(status, 0, sizeof(int), st));
-    IE_CK(cudaMemsetAsync(A, 0, (size_t)mf * kNU * sizeof(double2), st));
-    IE_CK(cudaMemsetAsync(V, 0, (size_t)mf * kNU * sizeof(double2), st));
-
-    sample_matrix_kernel<<<(s.ns * kSites + 255) / 256, 256, 0, st>>>(s, A, mf, A0);
-    IE_CK_LAUNCH();
-    householder_qr_kernel<<<1, 1024, 0, st>>>(A, mf, m, spec->tikhonov, V, tau, status);
-    IE_CK_LAUNCH();
-    int h_status = 0;
-    IE_CK(cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    IE_CK(cudaStreamSynchronize(st));
-    if (h_status) return set_error("the uniform-dipole field matrix A is rank deficient"), IE_ERR_INVALID;
-    const size_t pinv_smem = (size_t)kPinvWarps * mf * sizeof(double2);
-    IE_CK(cudaFuncSetAttribute(pinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pinv_smem));
-    pinv_kernel<<<(m + kPinvWarps - 1) / kPinvWarps, 32 * kPinvWarps, pinv_smem, st>>>(A, V, tau, mf, m, Apinv);
-    IE_CK_LAUNCH();
-
-    const size_t map_smem = (size_t)kFunPerCta * (m + kNU) * sizeof(double2);
-    IE_CK(cudaFuncSetAttribute(map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)map_smem));
     const int64_t chunk = n_fun < kMapChunk ? n_fun : kMapChunk;
     int64_t max_dip = 0;
     for (int64_t f0 = 0; f0 < n_fun; f0 += chunk) {
         int64_t f1 = f0 + chunk < n_fun ? f0 + chunk : n_fun;
         max_dip = std::max(max_dip, fun_off[f1] - fun_off[f0]);
     }
-    int64_t *d_off;
-    double *d_pos, *d_res = nullptr;
-    double2 *d_mom, *d_P;
-    IE_TRY(sc.get(&d_off, (size_t)chunk + 1));
-    IE_TRY(sc.get(&d_pos, 3 * (size_t)max_dip));
-    IE_TRY(sc.get(&d_mom, 3 * (size_t)max_dip));
-    IE_TRY(sc.get(&d_P, (size_t)chunk * kNU));
-    if (residual) IE_TRY(sc.get(&d_res, (size_t)chunk));
+    Scratch sc;
+    {
+        size_t b = 2 * Scratch::round((size_t)mf * kNU * sizeof(double2)) +
+                   2 * Scratch::round((size_t)m * kNU * sizeof(double2)) + Scratch::round(kNU * sizeof(double)) +
+                   Scratch::round((kNU + 1) * sizeof(int)) + Scratch::round(((size_t)chunk + 1) * sizeof(int64_t)) +
+                   Scratch::round(3 * (size_t)max_dip * sizeof(double)) +
+                   Scratch::round(3 * (size_t)max_dip * sizeof(double2)) +
+                   Scratch::round((size_t)chunk * kNU * sizeof(double2));
+        if (residual) b += Scratch::round((size_t)chunk * sizeof(double));
+        IE_TRY(sc.reserve(b));
+    }
+    double2 *A = sc.get<double2>((size_t)mf * kNU), *V = sc.get<double2>((size_t)mf * kNU);
+    double2 *A0 = sc.get<double2>((size_t)m * kNU), *Apinv = sc.get<double2>((size_t)m * kNU);
+    double *tau = sc.get<double>(kNU);
+    int *flag = sc.get<int>(kNU + 1);
+    int64_t *d_off = sc.get<int64_t>((size_t)chunk + 1);
+    double *d_pos = sc.get<double>(3 * (size_t)max_dip);
+    double2 *d_mom = sc.get<double2>(3 * (size_t)max_dip);
+    double2 *d_P = sc.get<double2>((size_t)chunk * kNU);
+    double *d_res = residual ? sc.get<double>((size_t)chunk) : nullptr;
+    int *status = flag + kNU;
+    IE_CK(cudaMemsetAsync(flag, 0, (kNU + 1) * sizeof(int), st));
+
+    sample_matrix_kernel<<<(s.ns * kSites + 255) / 256, 256, 0, st>>>(s, A, mf, A0);
+    IE_CK_LAUNCH();
+    {   // its CTAs wait on one another: all of them resident
+        int mq = mf, md = m;
+        double tk = spec->tikhonov;
+        void *args[] = {&A, &A0, &mq, &md, &tk, &V, &tau, &flag, &Apinv, &status};
+        IE_CK(cudaLaunchCooperativeKernel((const void *)qr_kernel, dim3(kNU), dim3(kQrThreads), args, 0, st));
+        IE_CK_LAUNCH();
+    }
+    int h_status = 0;
+    IE_CK(cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    IE_CK(cudaStreamSynchronize(st));
+    if (h_status == 1) return set_error("the uniform-dipole field matrix A is rank deficient"), IE_ERR_INVALID;
+    if (h_status) return set_error("the factorisation gave up a bounded wait"), IE_ERR_TIMEOUT;
+    pinv_solve_kernel<<<m, 32, 0, st>>>(A, mf, Apinv);
+    IE_CK_LAUNCH();
+
+    const size_t map_smem = (size_t)kFunPerCta * (m + kNU) * sizeof(double2);
+    IE_CK(cudaFuncSetAttribute(map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)map_smem));
     std::vector<int64_t> off(chunk + 1);
     for (int64_t f0 = 0; f0 < n_fun; f0 += chunk) {
         const int64_t nf = std::min(chunk, n_fun - f0);
