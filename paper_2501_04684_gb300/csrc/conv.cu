@@ -23,8 +23,8 @@
 // odd along each axis), rounded once to FP32, with 1 / (L_x L_y L_z) folded in.
 //
 // Cost: O(L^3 log L) instead of 192^2 multiply-adds per far pair.  Measured far part of one
-// IE_FULL product: 0.50 ms on the 32^3 shell (L = 256: x 26, y 52, z 340, y back 49, x back
-// 28 us) against 17.7 ms (FP16X3) and 150 ms (FP32) of the block products; 0.067 ms on the
+// IE_FULL product: 0.39 ms on the 32^3 shell (L = 256: x 26, y 52, z 231, y back 49, x back
+// 28 us) against 17.7 ms (FP16X3) and 150 ms (FP32) of the block products; 0.064 ms on the
 // 16^3 shell (L = 128) against 1.5 and 12.2 ms.
 #include <algorithm>
 #include <array>
@@ -184,7 +184,7 @@ struct ConvArgs {
     float2 *Y;                  // [rhs][nbox][192]
     float2 *A, *B;              // per column a_col / b_col elements
     int64_t a_col, b_col;
-    const float4 *K;            // [kz][ky][kx][xx xy | xz yy | yz zz], octant
+    const float4 *K;            // [xx xy | xz yy | yz zz][kz][ky][kx], octant
     const int32_t *slot;        // [scatterer][Ez][Ey][Ex] box, or -1
     const int32_t *cols;        // [scatterer] right-hand sides it takes part with
     const float2 *twx, *twy, *twz;   // exp(-2 pi i j / L)
@@ -372,8 +372,16 @@ __device__ __forceinline__ void cmac(float2 &d, float2 a, float2 b) {
 // z pass of one (ky, kx tile): transform, tensor product, transform back, in place.  Blocks
 // of mirrored (ky, kx) run next to each other, so that the octant of K^ they share is read
 // from device memory once.
-template <int R1, int R2>
-__global__ void __launch_bounds__(kW *R2) conv_z_kernel(const ConvArgs a) {
+//
+// Bound by latency (loads of K^ and of the lines) at the occupancy that shared memory (24 L kW
+// bytes) and registers (three components of an R2-point sum) leave: 46% of the issue slots at L
+// = 256 with two CTAs per SM, 231 us on the 32^3 shell; one CTA per SM and K^ as 48-byte records
+// took 340 us.  Up to L = 192 the registers hold K^ points and lines ahead (16^3 shell 32 -> 29
+// us, 4^3 grid 9.8 -> 6.4); at L = 256 they do not (lines ahead 318 us, R1 = 32 with K^ ahead but
+// half the threads 254, tiles of 8 lines 253).
+// PFMAX: points of K^ fetched ahead of their use; AHEAD: the three components' lines too.
+template <int R1, int R2, int PFMAX, bool AHEAD, int CTAS>
+__global__ void __launch_bounds__(kW *R2, CTAS) conv_z_kernel(const ConvArgs a) {
     if (a.gate && *a.gate == 0) return;
     constexpr int L = R1 * R2, NT = kW * R2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -387,33 +395,59 @@ __global__ void __launch_bounds__(kW *R2) conv_z_kernel(const ConvArgs a) {
     const int ky = (blockIdx.y & 1) ? a.Ly - 1 - (blockIdx.y >> 1) : (blockIdx.y >> 1);
     const int64_t plane = (int64_t)a.Ly * a.Lx;
     float2 *B = a.B + blockIdx.z * a.b_col + (int64_t)ky * a.Lx + kx;
-    for (int i = threadIdx.x; i < L; i += NT) tw[i] = a.twz[i];
-    __syncthreads();
-    for (int c = 0; c < 3; ++c) {
-        float2 v[R1];
+    auto load = [&](int c, float2(&u)[R1 / 2]) {
         unroll<R1 / 2>([&](auto i) {
             const int z = R2 * i + b0;
-            v[i] = z < nz ? B[((int64_t)c * nz + z) * plane] : make_float2(0.f, 0.f);
+            u[i] = z < nz ? B[(int64_t)(c * nz + z) * plane] : make_float2(0.f, 0.f);
         });
+    };
+    auto first = [&](int c, const float2(&u)[R1 / 2]) {
+        float2 v[R1];
+        unroll<R1 / 2>([&](auto i) { v[i] = u[i]; });
         dft_half_in<R1>(v);
         unroll<R1>([&](auto k) { S[((c * R1 + k) * R2 + b0) * kW + w] = cmulf(v[k], tw[b0 * k]); });
+    };
+    if constexpr (AHEAD) {      // all three components' loads in flight together
+        float2 u[3][R1 / 2];
+        unroll<3>([&](auto c) { load(c, u[c]); });
+        for (int i = threadIdx.x; i < L; i += NT) tw[i] = a.twz[i];
+        __syncthreads();
+        unroll<3>([&](auto c) { first(c, u[c]); });
+    } else {
+        for (int i = threadIdx.x; i < L; i += NT) tw[i] = a.twz[i];
+        __syncthreads();
+#pragma unroll 1
+        for (int c = 0; c < 3; ++c) {
+            float2 u[R1 / 2];
+            load(c, u);
+            first(c, u);
+        }
     }
     __syncthreads();
     const int ax = 2 * kx > a.Lx ? a.Lx - kx : kx, ay = 2 * ky > a.Ly ? a.Ly - ky : ky;
     const float sx = 2 * kx > a.Lx ? -1.f : 1.f, sy = 2 * ky > a.Ly ? -1.f : 1.f;
     const int mx = a.Lx / 2 + 1, my = a.Ly / 2 + 1;
+    const int64_t kpart = (int64_t)(L / 2 + 1) * my * mx;
+    constexpr int PF = R2 < PFMAX ? R2 : PFMAX;
     for (int k1 = b0; k1 < R1; k1 += R2) {
+        float4 f[PF][3];
+        auto fetch = [&](int k2, float4(&g)[3]) {
+            const int kz = k1 + R1 * k2;
+            const int az = 2 * kz > L ? L - kz : kz;
+            const float4 *K = a.K + ((int64_t)az * my + ay) * mx + ax;
+            g[0] = __ldg(K), g[1] = __ldg(K + kpart), g[2] = __ldg(K + 2 * kpart);
+        };
+        unroll<PF>([&](auto i) { fetch(i, f[i]); });
         float2 v[3][R2];
         unroll<3>([&](auto c) {
             unroll<R2>([&](auto b) { v[c][b] = S[((c * R1 + k1) * R2 + b) * kW + w]; });
             dft<R2, -1>(v[c]);
         });
         unroll<R2>([&](auto k2) {
-            const int kz = k1 + R1 * k2;
-            const int az = 2 * kz > L ? L - kz : kz;
-            const float sz = 2 * kz > L ? -1.f : 1.f;
-            const float4 *K = a.K + (((int64_t)az * my + ay) * mx + ax) * 3;
-            const float4 f0 = __ldg(K), f1 = __ldg(K + 1), f2 = __ldg(K + 2);
+            constexpr int at = decltype(k2)::value % PF;
+            const float sz = 2 * (k1 + R1 * k2) > L ? -1.f : 1.f;
+            const float4 f0 = f[at][0], f1 = f[at][1], f2 = f[at][2];
+            if constexpr (decltype(k2)::value + PF < R2) fetch(k2 + PF, f[at]);
             const float sxy = sx * sy, sxz = sx * sz, syz = sy * sz;
             const float2 xx = make_float2(f0.x, f0.y), xy = make_float2(sxy * f0.z, sxy * f0.w);
             const float2 xz = make_float2(sxz * f1.x, sxz * f1.y), yy = make_float2(f1.z, f1.w);
@@ -434,6 +468,7 @@ __global__ void __launch_bounds__(kW *R2) conv_z_kernel(const ConvArgs a) {
         });
     }
     __syncthreads();
+#pragma unroll 1
     for (int c = 0; c < 3; ++c) {
         float2 v[R1];
         unroll<R1>([&](auto k) { v[k] = S[((c * R1 + k) * R2 + b0) * kW + w]; });
@@ -449,6 +484,11 @@ __global__ void __launch_bounds__(kW *R2) conv_z_kernel(const ConvArgs a) {
 #define IE_CONV_SIZES(F) \
     F(16, 4, 4) F(32, 8, 4) F(48, 12, 4) F(64, 8, 8) F(96, 12, 8) F(128, 16, 8) F(192, 24, 8) F(256, 16, 16) \
     F(384, 24, 16) F(512, 32, 16)
+// z lines: K^ points ahead, lines ahead, CTAs per SM (shared memory and registers)
+#define IE_CONV_ZSIZES(F)                                                                                    \
+    F(16, 4, 4, 4, true, 8) F(32, 8, 4, 4, true, 8) F(48, 12, 4, 4, true, 8) F(64, 8, 8, 4, true, 4)         \
+    F(96, 12, 8, 4, true, 4) F(128, 16, 8, 4, true, 4) F(192, 24, 8, 4, false, 3) F(256, 16, 16, 1, false, 2) \
+    F(384, 24, 16, 2, false, 1) F(512, 32, 16, 2, false, 1)
 
 template <int R1, int R2>
 constexpr size_t x_smem() { return (size_t)(3 * XTile<R2>::rows * x_line<R1, R2>() + R1 * R2) * sizeof(float2); }
@@ -516,7 +556,7 @@ __global__ void conv_axis_kernel(const double2 *__restrict__ in, double2 *__rest
     auto put = [&](int kk, double re, double im) {
         const int64_t at = (c / inner) * (K * inner) + kk * inner + c % inner;
         if (out32)
-            out32[6 * at] = make_float2((float)(scale * re), (float)(scale * im));
+            out32[2 * at] = make_float2((float)(scale * re), (float)(scale * im));
         else
             out[at] = make_double2(re, im);
     };
@@ -543,7 +583,6 @@ ie_status set_attr() {
     IE_CK(cudaFuncSetAttribute(conv_y_kernel<R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)y_smem<R1, R2>()));
     IE_CK(cudaFuncSetAttribute(conv_yback_kernel<R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)y_smem<R1, R2>()));
-    IE_CK(cudaFuncSetAttribute(conv_z_kernel<R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)z_smem<R1, R2>()));
     return IE_OK;
 }
 
@@ -552,6 +591,11 @@ ie_status set_attr() {
 ie_status prepare_conv() {
 #define IE_ATTR(L, R1, R2) IE_TRY((set_attr<R1, R2>()));
     IE_CONV_SIZES(IE_ATTR)
+#undef IE_ATTR
+#define IE_ATTR(L, R1, R2, PF, AHEAD, CTAS)                                                                         \
+    IE_CK(cudaFuncSetAttribute(conv_z_kernel<R1, R2, PF, AHEAD, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                               (int)z_smem<R1, R2>()));
+    IE_CONV_ZSIZES(IE_ATTR)
 #undef IE_ATTR
     return IE_OK;
 }
@@ -566,7 +610,7 @@ constexpr double kConvKa = 0.75;
 // place the line for scatterers that are sparse in their bounding box; measured with random
 // boxes on grids of 3^3 to 64^3, e.g. 600 boxes on 24^3 249 us here against 441 us (FP16X3),
 // 200 boxes 243 against 179; 1,200 boxes on 64^3 4.1 ms against 3.0 ms.
-constexpr double kPointNs = 0.033, kPairNs16 = 0.7, kBlockNs16 = 49, kPairNs32 = 6.0, kBlockNs32 = 270;
+constexpr double kPointNs = 0.03, kPairNs16 = 0.7, kBlockNs16 = 49, kPairNs32 = 6.0, kBlockNs32 = 270;
 // A far product alone also takes the adjacent pairs off (a second kernel's chain): below this
 // many far pairs the block product is the shorter chain (5,650 pairs 87 against 105 us, 9,356
 // pairs 140 against 106 us in FP32).
@@ -706,7 +750,8 @@ ie_status build_khat(ie_plan p, ConvClass &c, cudaStream_t st) {
                 IE_CK_LAUNCH();
                 axis(1, t1, t0, nullptr, n[0], K[2] * n[0]);
                 IE_CK_LAUNCH();
-                axis(0, t0, nullptr, reinterpret_cast<float2 *>(c.d_K) + comp, 1, K[2] * K[1]);
+                axis(0, t0, nullptr, reinterpret_cast<float2 *>(c.d_K + (comp / 2) * K[2] * K[1] * K[0]) + comp % 2, 1,
+                     K[2] * K[1]);
                 IE_CK_LAUNCH();
             }
         return IE_OK;
@@ -797,9 +842,9 @@ ie_status launch_conv(ie_plan p, const float2 *X, float2 *Y, int nrhs, cudaStrea
             switch (a.Ly) { IE_CONV_SIZES(IE_CASE) }
 #undef IE_CASE
             IE_CK_LAUNCH();
-#define IE_CASE(L, R1, R2) \
-    case L: conv_z_kernel<R1, R2><<<zgrid, kW * R2, z_smem<R1, R2>(), st>>>(a); break;
-            switch (a.Lz) { IE_CONV_SIZES(IE_CASE) }
+#define IE_CASE(L, R1, R2, PF, AHEAD, CTAS) \
+    case L: conv_z_kernel<R1, R2, PF, AHEAD, CTAS><<<zgrid, kW * R2, z_smem<R1, R2>(), st>>>(a); break;
+            switch (a.Lz) { IE_CONV_ZSIZES(IE_CASE) }
 #undef IE_CASE
             IE_CK_LAUNCH();
 #define IE_CASE(L, R1, R2) \
