@@ -750,6 +750,7 @@ static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream,
     for (int b = 0; b < p->nbox; ++b) {
         p->nb[b] = pr->nb ? pr->nb[b] : kNU;
         p->off[b + 1] = p->off[b] + p->nb[b];
+        p->max_nb = std::max(p->max_nb, p->nb[b]);
     }
     p->n = p->off[p->nbox];
     p->ngroups = n_groups_of(pr);

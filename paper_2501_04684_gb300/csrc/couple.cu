@@ -144,13 +144,6 @@ struct SmemNear {
 };
 static_assert(sizeof(float2) * kNU * kNearJ == sizeof(float2) * 2 * kNearKC * kNU, "W overlays the chunks");
 
-// (hi, lo) += x
-__device__ __forceinline__ void add2(float &hi, float &lo, float x) {
-    const float s = hi + x, bb = s - hi;
-    lo += (hi - (s - bb)) + (x - bb);
-    hi = s;
-}
-
 __global__ void __launch_bounds__(kNearThreads)
 near_blocks_kernel(const float2 *__restrict__ Cnear,     // [27 or 54][k][m], index by e
                    const int32_t *__restrict__ ijk, const int32_t *__restrict__ nb, const int64_t *__restrict__ off,
@@ -228,8 +221,8 @@ near_blocks_kernel(const float2 *__restrict__ Cnear,     // [27 or 54][k][m], in
                     for (int i = 0; i < 6; ++i)
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            add2(hi[i][j].x, lo[i][j].x, acc[i][j].x);
-                            add2(hi[i][j].y, lo[i][j].y, acc[i][j].y);
+                            two_float_add(hi[i][j].x, lo[i][j].x, acc[i][j].x);
+                            two_float_add(hi[i][j].y, lo[i][j].y, acc[i][j].y);
                             acc[i][j] = make_float2(0.f, 0.f);
                         }
                 }
@@ -264,8 +257,8 @@ near_blocks_kernel(const float2 *__restrict__ Cnear,     // [27 or 54][k][m], in
                     }
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
-                        add2(h[r].x, l[r].x, q[r].x);
-                        add2(h[r].y, l[r].y, q[r].y);
+                        two_float_add(h[r].x, l[r].x, q[r].x);
+                        two_float_add(h[r].y, l[r].y, q[r].y);
                     }
                 }
 #pragma unroll

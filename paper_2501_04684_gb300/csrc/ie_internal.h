@@ -86,6 +86,14 @@ __device__ inline void dyad_fp64(double k, double eta, double Rx, double Ry, dou
         }
 }
 
+// (hi, lo) += x without losing the rounding of the sum: FP32 chunk sums kept to twice FP32's
+// digits at FP32 rate (an FP64 addition takes the issue time of 64 FP32 ones on this GPU).
+__device__ __forceinline__ void two_float_add(float &hi, float &lo, float x) {
+    const float s = hi + x, b = s - hi;
+    lo += (hi - (s - b)) + (x - b);
+    hi = s;
+}
+
 void set_error(const char *fmt, ...);
 const char *last_error();
 
@@ -190,6 +198,7 @@ struct ie_plan_s {
     std::vector<int32_t> box_group;    // nbox scatterer of each box
     std::vector<int32_t> h_src;        // source box of every far pair (kept only with gnrhs)
     std::vector<int32_t> ijk, nb;
+    int max_nb = 0;                    // largest nb
     std::vector<int64_t> off;          // nbox + 1
 
     // device geometry and mapping
