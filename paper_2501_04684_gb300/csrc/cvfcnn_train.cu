@@ -12,12 +12,19 @@
 // Layout: one CTA per network (persistent over networks), 256 threads; an Adam step
 // sums the gradients of `minibatches` minibatches of 32 samples, each held in shared
 // memory in turn:
-//   X  [192][33]  inputs x / s (column j = sample j; rows padded to 33 against bank
-//                 conflicts)
-//   R  [192][33]  target G x / (s g) (g = max |G| of the block, so the weights the
+//   X  [192][34]  inputs x / s (column j = sample j; rows of 272 bytes: 16-byte reads along
+//                 a row and down the rows are free of bank conflicts)
+//   R  [192][34]  target G x / (s g) (g = max |G| of the block, so the weights the
 //                 optimiser sees are of order one), then the output residual
-//   Z  [64][33]   hidden pre-activations, then the back-propagated hidden gradient
-//   Hh [64][33]   hidden activations
+//   Z  [64][34]   hidden pre-activations, then the back-propagated hidden gradient
+//   Hh [64][34]   hidden activations
+//   A              two chunks of the matrix a product reads from global memory (cp.async)
+// The six products of a minibatch run on register tiles: 6 x 4 outputs per thread for the
+// 192-row ones (target, output layer), 4 x 2 for the 64-row ones (hidden layer, hidden
+// gradient), 7 x 6 for the two weight gradients.  FP32 rate bound, one CTA (two warps per
+// scheduler) per SM: 192 x 192 + 5 x 192 H complex multiply-adds per sample, 0.17 ms per step
+// of 128 samples at the peak rate for H = 50; 0.43 ms measured (1.0 ms with operands
+// read per multiply-add from global memory and one gradient entry per thread at a time).
 // Weights and Adam moments live in global memory (L2-resident while the CTA trains):
 // W1 [64][192], W2T [64][192] (W2 transposed), b1 [64], b2 [192]; rows h >= H stay zero.
 // Per step: x from a counter-based hash (the generator is stated below), s = max |x_u|,
@@ -39,7 +46,10 @@ namespace ie {
 namespace {
 
 constexpr int kTB = 32;             // minibatch
-constexpr int kTP = kTB + 1;        // padded row length (float2)
+constexpr int kTP = kTB + 2;        // padded row length (float2)
+constexpr int kTK = 16;             // rows of a chunk of a 192-row product's matrix
+constexpr int kTC = 32;             // columns of a chunk of a 64-row product's matrix
+constexpr int kTCP = kTC + 2;
 constexpr int kTrainThreads = 256;
 constexpr int kTestSamples = 64;
 constexpr int kWElems = kCvHp * kNU;                    // W1 or W2T
@@ -51,6 +61,10 @@ struct SmemTrain {
     float2 R[kNU][kTP];
     float2 Z[kCvHp][kTP];
     float2 Hh[kCvHp][kTP];
+    union {
+        float2 big[2][kTK][kNU];
+        float2 hid[2][kCvHp][kTCP];
+    } A;
     float inv_s[kTB];
     float red[kTrainThreads / 32];
     float err[kTB];
@@ -128,81 +142,166 @@ __device__ void make_inputs(SmemTrain &S, const TrainArgs &a, uint32_t net, uint
     __syncthreads();
 }
 
-// R[m][j] = sum_k G[m][k] X[k][j] / g  (thread: 4 columns, 6 rows)
+__device__ __forceinline__ void copy16(void *smem, const void *gmem) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void copies_end() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
+// acc[i][c] += sum_k A[k][row i] B[k][column c], k < K <= 192, A [K][192] in global memory
+// (whole chunks of 16 rows readable), B in shared memory.  Thread: rows 2 tm, + 1 (+ 64 i),
+// columns 4 tn .. + 3, tm = t / 8, tn = t mod 8.  Ends with a barrier.
+__device__ __forceinline__ void product192(SmemTrain &S, const float2 *A, int K, const float2 (*B)[kTP],
+                                           float2 (&acc)[6][4]) {
+    const int t = threadIdx.x, tm = t >> 3, tn = t & 7, chunks = (K + kTK - 1) / kTK;
+    auto load = [&](int c) {
+        const float4 *g = reinterpret_cast<const float4 *>(A + (size_t)c * kTK * kNU);
+        float4 *d = reinterpret_cast<float4 *>(&S.A.big[c & 1][0][0]);
+#pragma unroll
+        for (int i = 0; i < kTK * kNU / 2 / kTrainThreads; ++i) copy16(d + t + i * kTrainThreads, g + t + i * kTrainThreads);
+        copies_end();
+    };
+    load(0);
+    for (int c = 0; c < chunks; ++c) {
+        if (c + 1 < chunks) {
+            load(c + 1);
+            copies_wait<1>();
+        } else {
+            copies_wait<0>();
+        }
+        __syncthreads();
+        const int kn = min(kTK, K - c * kTK);
+#pragma unroll 2
+        for (int k = 0; k < kn; ++k) {
+            float2 a[6], b[4];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const float4 v = *reinterpret_cast<const float4 *>(&S.A.big[c & 1][k][2 * tm + 64 * i]);
+                a[2 * i] = make_float2(v.x, v.y);
+                a[2 * i + 1] = make_float2(v.z, v.w);
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float4 v = *reinterpret_cast<const float4 *>(&B[c * kTK + k][4 * tn + 2 * i]);
+                b[2 * i] = make_float2(v.x, v.y);
+                b[2 * i + 1] = make_float2(v.z, v.w);
+            }
+#pragma unroll
+            for (int i = 0; i < 6; ++i)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) cfma(acc[i][q], a[i], b[q]);
+        }
+        __syncthreads();
+    }
+}
+__device__ __forceinline__ int row192(int i) { return 2 * (threadIdx.x >> 3) + 64 * (i >> 1) + (i & 1); }
+__device__ __forceinline__ int col192(int q) { return 4 * (threadIdx.x & 7) + q; }
+
+// acc[r][c] = sum_k A[row r][k] B[k][column c] (CONJ: conj(A)), k < 192, A [64][192] in global
+// memory, B in shared memory.  Thread: rows t / 16 + 16 r (below H), columns 2 (t mod 16), + 1.
+// Ends with a barrier.
+template <bool CONJ>
+__device__ __forceinline__ void product64(SmemTrain &S, const float2 *A, int H, const float2 (*B)[kTP],
+                                          float2 (&acc)[4][2]) {
+    const int t = threadIdx.x, hg = t >> 4, jp = 2 * (t & 15);
+    auto load = [&](int c) {
+#pragma unroll
+        for (int i = 0; i < kCvHp * kTC / 2 / kTrainThreads; ++i) {
+            const int e = t + i * kTrainThreads, h = e / (kTC / 2), k = 2 * (e % (kTC / 2));
+            copy16(&S.A.hid[c & 1][h][k], A + (size_t)h * kNU + c * kTC + k);
+        }
+        copies_end();
+    };
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
+    load(0);
+    for (int c = 0; c < kNU / kTC; ++c) {
+        if (c + 1 < kNU / kTC) {
+            load(c + 1);
+            copies_wait<1>();
+        } else {
+            copies_wait<0>();
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int k = 0; k < kTC; k += 2) {
+            const float4 x0 = *reinterpret_cast<const float4 *>(&B[c * kTC + k][jp]);
+            const float4 x1 = *reinterpret_cast<const float4 *>(&B[c * kTC + k + 1][jp]);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (hg + 16 * r < H) {
+                    const float4 w = *reinterpret_cast<const float4 *>(&S.A.hid[c & 1][hg + 16 * r][k]);
+                    const float2 b[2][2] = {{make_float2(x0.x, x0.y), make_float2(x0.z, x0.w)},
+                                            {make_float2(x1.x, x1.y), make_float2(x1.z, x1.w)}};
+                    const float2 a[2] = {make_float2(w.x, w.y), make_float2(w.z, w.w)};
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            if (CONJ) {
+                                acc[r][q].x = fmaf(a[e].x, b[e][q].x, fmaf(a[e].y, b[e][q].y, acc[r][q].x));
+                                acc[r][q].y = fmaf(a[e].x, b[e][q].y, fmaf(-a[e].y, b[e][q].x, acc[r][q].y));
+                            } else {
+                                cfma(acc[r][q], a[e], b[e][q]);
+                            }
+                        }
+                }
+        }
+        __syncthreads();
+    }
+}
+
+// R[m][j] = sum_k G[m][k] X[k][j] / g
 __device__ void teacher(SmemTrain &S, const float2 *__restrict__ G, float ginv) {
-    const int t = threadIdx.x, j0 = 4 * (t & 7), mr = t >> 3;
     float2 acc[6][4];
 #pragma unroll
     for (int i = 0; i < 6; ++i)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[i][c] = make_float2(0.f, 0.f);
-    for (int k = 0; k < kNU; ++k) {
-        float2 g[6], x[4];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) g[i] = __ldg(G + (size_t)k * kNU + mr + 32 * i);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) x[c] = S.X[k][j0 + c];
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) cfma(acc[i][c], g[i], x[c]);
-    }
+    product192(S, G, kNU, S.X, acc);
 #pragma unroll
     for (int i = 0; i < 6; ++i)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) S.R[mr + 32 * i][j0 + c] = make_float2(acc[i][c].x * ginv, acc[i][c].y * ginv);
+        for (int c = 0; c < 4; ++c) S.R[row192(i)][col192(c)] = make_float2(acc[i][c].x * ginv, acc[i][c].y * ginv);
 }
 
-// Z = W1 X + b1, Hh = relu(Z) (thread: column j, rows hr + 8 i)
-__device__ void forward_hidden(SmemTrain &S, const float2 *__restrict__ W1, const float2 *__restrict__ b1, int H) {
-    const int t = threadIdx.x, j = t & 31, hr = t >> 5;
-    float2 acc[8];
+// Z = W1 X + b1, Hh = relu(Z)
+__device__ void forward_hidden(SmemTrain &S, const float2 *W1, const float2 *b1, int H) {
+    float2 acc[4][2];
+    product64<false>(S, W1, H, S.X, acc);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] = make_float2(0.f, 0.f);
-    for (int k = 0; k < kNU; ++k) {
-        const float2 x = S.X[k][j];
+    for (int r = 0; r < 4; ++r) {
+        const int h = (threadIdx.x >> 4) + 16 * r;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (hr + 8 * i < H) cfma(acc[i], W1[(size_t)(hr + 8 * i) * kNU + k], x);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int h = hr + 8 * i;
-        float2 z = make_float2(0.f, 0.f);
-        if (h < H) z = make_float2(acc[i].x + b1[h].x, acc[i].y + b1[h].y);
-        S.Z[h][j] = z;
-        S.Hh[h][j] = make_float2(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f));
+        for (int q = 0; q < 2; ++q) {
+            const int j = 2 * (threadIdx.x & 15) + q;
+            float2 z = make_float2(0.f, 0.f);
+            if (h < H) z = make_float2(acc[r][q].x + b1[h].x, acc[r][q].y + b1[h].y);
+            S.Z[h][j] = z;
+            S.Hh[h][j] = make_float2(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f));
+        }
     }
 }
 
-// out[m][j] = W2 Hh + b2 (thread: 4 columns, 6 rows); mode 0: R = c (out - R);
-// mode 1: per-sample |out - R|^2 and |R|^2 into S.err / S.enorm (test set)
-__device__ void forward_output(SmemTrain &S, const float2 *__restrict__ W2T, const float2 *__restrict__ b2, int H,
-                               float c, int mode) {
-    const int t = threadIdx.x, j0 = 4 * (t & 7), mr = t >> 3;
+// out[m][j] = W2 Hh + b2; mode 0: R = c (out - R); mode 1: per-sample |out - R|^2 and |R|^2
+// into S.err / S.enorm (test set)
+__device__ void forward_output(SmemTrain &S, const float2 *W2T, const float2 *b2, int H, float c, int mode) {
     float2 acc[6][4];
 #pragma unroll
     for (int i = 0; i < 6; ++i)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[i][q] = b2[mr + 32 * i];
-    for (int k = 0; k < H; ++k) {
-        float2 w[6], h[4];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) w[i] = W2T[(size_t)k * kNU + mr + 32 * i];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) h[q] = S.Hh[k][j0 + q];
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) cfma(acc[i][q], w[i], h[q]);
-    }
+        for (int q = 0; q < 4; ++q) acc[i][q] = b2[row192(i)];
+    product192(S, W2T, H, S.Hh, acc);
     if (mode == 0) {
-        __syncthreads();   // every thread has read what it needs before R changes meaning
 #pragma unroll
         for (int i = 0; i < 6; ++i)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                float2 &r = S.R[mr + 32 * i][j0 + q];
+                float2 &r = S.R[row192(i)][col192(q)];
                 r = make_float2(c * (acc[i][q].x - r.x), c * (acc[i][q].y - r.y));
             }
     } else {
@@ -211,16 +310,64 @@ __device__ void forward_output(SmemTrain &S, const float2 *__restrict__ W2T, con
         for (int i = 0; i < 6; ++i)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float2 r = S.R[mr + 32 * i][j0 + q];
+                const float2 r = S.R[row192(i)][col192(q)];
                 const float dx = acc[i][q].x - r.x, dy = acc[i][q].y - r.y;
                 e[q] += dx * dx + dy * dy;
                 n[q] += r.x * r.x + r.y * r.y;
             }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            atomicAdd(&S.err[j0 + q], e[q]);
-            atomicAdd(&S.enorm[j0 + q], n[q]);
+            atomicAdd(&S.err[col192(q)], e[q]);
+            atomicAdd(&S.enorm[col192(q)], n[q]);
         }
+    }
+}
+
+// g[r][i] = sum_j a_rj conj(b_ij) over the 32 samples for rows h = warp + 8 r < H of `rows` and
+// entries u = lane + 32 i of `cols`; swap: the entries are the rows' conjugates' partner, i.e.
+// sum_j cols[u][j] conj(rows[h][j]).
+template <bool SWAP, class F>
+__device__ __forceinline__ void gradient(const float2 (*rows)[kTP], const float2 (*cols)[kTP], int H, F use) {
+    constexpr int kR = kCvHp / 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // two halves of the rows: 4 x 6 sums in registers at a time
+#pragma unroll 1
+    for (int r0 = 0; r0 < kR; r0 += kR / 2) {
+        if (warp + 8 * r0 >= H) break;
+        float2 g[kR / 2][kNU / 32];
+#pragma unroll
+        for (int r = 0; r < kR / 2; ++r)
+#pragma unroll
+            for (int i = 0; i < kNU / 32; ++i) g[r][i] = make_float2(0.f, 0.f);
+#pragma unroll 1
+        for (int j = 0; j < kTB; j += 2) {
+            float4 b[kNU / 32];
+#pragma unroll
+            for (int i = 0; i < kNU / 32; ++i) b[i] = *reinterpret_cast<const float4 *>(&cols[lane + 32 * i][j]);
+#pragma unroll
+            for (int r = 0; r < kR / 2; ++r)
+                if (warp + 8 * (r0 + r) < H) {
+                    const float4 h = *reinterpret_cast<const float4 *>(&rows[warp + 8 * (r0 + r)][j]);
+#pragma unroll
+                    for (int i = 0; i < kNU / 32; ++i) {
+                        float2 &q = g[r][i];
+                        if (SWAP) {         // cols conj(rows)
+                            q.x = fmaf(b[i].x, h.x, fmaf(b[i].y, h.y, q.x));
+                            q.y = fmaf(b[i].y, h.x, fmaf(-b[i].x, h.y, q.y));
+                            q.x = fmaf(b[i].z, h.z, fmaf(b[i].w, h.w, q.x));
+                            q.y = fmaf(b[i].w, h.z, fmaf(-b[i].z, h.w, q.y));
+                        } else {            // rows conj(cols)
+                            q.x = fmaf(h.x, b[i].x, fmaf(h.y, b[i].y, q.x));
+                            q.y = fmaf(h.y, b[i].x, fmaf(-h.x, b[i].y, q.y));
+                            q.x = fmaf(h.z, b[i].z, fmaf(h.w, b[i].w, q.x));
+                            q.y = fmaf(h.w, b[i].z, fmaf(-h.z, b[i].w, q.y));
+                        }
+                    }
+                }
+        }
+#pragma unroll
+        for (int r = 0; r < kR / 2; ++r)
+            if (warp + 8 * (r0 + r) < H) use((warp + 8 * (r0 + r)) * kNU + lane, g[r]);
     }
 }
 
@@ -242,6 +389,29 @@ __device__ __forceinline__ void accumulate(float2 &p, float2 &m, float2 &v, floa
         adam(p, m, v, g, lr_t, c1, c2);
     else
         gs = g;
+}
+
+// The same for the six entries at idx + 32 i of one row: all their reads are in flight before
+// the first store.
+__device__ __forceinline__ void accumulate_row(float2 *P, float2 *M, float2 *V, float2 *Gs, int idx,
+                                               const float2 (&g)[kNU / 32], bool first, bool last, float lr_t, float c1,
+                                               float c2) {
+    constexpr int N = kNU / 32;
+    float2 gs[N], p[N], m[N], v[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        if (!first) gs[i] = Gs[idx + 32 * i];
+        if (last) p[i] = P[idx + 32 * i], m[i] = M[idx + 32 * i], v[i] = V[idx + 32 * i];
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) accumulate(p[i], m[i], v[i], gs[i], g[i], first, last, lr_t, c1, c2);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        if (last)
+            P[idx + 32 * i] = p[i], M[idx + 32 * i] = m[i], V[idx + 32 * i] = v[i];
+        else
+            Gs[idx + 32 * i] = gs[i];
+    }
 }
 
 __global__ void __launch_bounds__(kTrainThreads, 1) cvfcnn_train_kernel(const TrainArgs a) {
@@ -331,42 +501,21 @@ __global__ void __launch_bounds__(kTrainThreads, 1) cvfcnn_train_kernel(const Tr
             __syncthreads();
             // hidden gradient with the old W2: dH = W2^H R, then dZ = dH through the ReLU (into Z)
             {
-                const int j = t & 31, hr = t >> 5;
-                float2 acc[8];
+                float2 acc[4][2];
+                product64<true>(S, W2T, H, S.R, acc);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) acc[i] = make_float2(0.f, 0.f);
-                for (int m = 0; m < kNU; ++m) {
-                    const float2 r = S.R[m][j];
+                for (int r = 0; r < 4; ++r)
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (hr + 8 * i < H) {
-                            const float2 w = W2T[(size_t)(hr + 8 * i) * kNU + m];
-                            // conj(w) r
-                            acc[i].x = fmaf(w.x, r.x, fmaf(w.y, r.y, acc[i].x));
-                            acc[i].y = fmaf(w.x, r.y, fmaf(-w.y, r.x, acc[i].y));
-                        }
-                }
-                __syncthreads();
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int h = hr + 8 * i;
-                    const float2 z = S.Z[h][j];
-                    S.Z[h][j] = make_float2(z.x > 0.f ? acc[i].x : 0.f, z.y > 0.f ? acc[i].y : 0.f);
-                }
+                    for (int q = 0; q < 2; ++q) {
+                        const int h = (t >> 4) + 16 * r, j = 2 * (t & 15) + q;
+                        const float2 z = S.Z[h][j];
+                        S.Z[h][j] = make_float2(z.x > 0.f ? acc[r][q].x : 0.f, z.y > 0.f ? acc[r][q].y : 0.f);
+                    }
             }
             // W2 (transposed) and b2: dW2T[k][m] = sum_j R[m][j] conj(Hh[k][j])
-            for (int idx = t; idx < H * kNU; idx += kTrainThreads) {
-                const int k = idx / kNU, m = idx % kNU;
-                float2 g = make_float2(0.f, 0.f);
-#pragma unroll 8
-                for (int j = 0; j < kTB; ++j) {
-                    const float2 r = S.R[m][j], h = S.Hh[k][j];
-                    g.x = fmaf(r.x, h.x, fmaf(r.y, h.y, g.x));
-                    g.y = fmaf(r.y, h.x, fmaf(-r.x, h.y, g.y));
-                }
-                accumulate(W2T[idx], M[kWElems + idx], V[kWElems + idx], Gs[kWElems + idx], g, first, last, lr_t, c1,
-                           c2);
-            }
+            gradient<true>(S.Hh, S.R, H, [&](int idx, const float2 (&g)[kNU / 32]) {
+                accumulate_row(P, M, V, Gs, kWElems + idx, g, first, last, lr_t, c1, c2);
+            });
             for (int m = t; m < kNU; m += kTrainThreads) {
                 float2 g = make_float2(0.f, 0.f);
                 for (int j = 0; j < kTB; ++j) g = make_float2(g.x + S.R[m][j].x, g.y + S.R[m][j].y);
@@ -375,17 +524,9 @@ __global__ void __launch_bounds__(kTrainThreads, 1) cvfcnn_train_kernel(const Tr
             }
             __syncthreads();
             // W1 and b1: dW1[h][u] = sum_j dZ[h][j] conj(X[u][j])
-            for (int idx = t; idx < H * kNU; idx += kTrainThreads) {
-                const int h = idx / kNU, u = idx % kNU;
-                float2 g = make_float2(0.f, 0.f);
-#pragma unroll 8
-                for (int j = 0; j < kTB; ++j) {
-                    const float2 d = S.Z[h][j], x = S.X[u][j];
-                    g.x = fmaf(d.x, x.x, fmaf(d.y, x.y, g.x));
-                    g.y = fmaf(d.y, x.x, fmaf(-d.x, x.y, g.y));
-                }
-                accumulate(W1[idx], M[idx], V[idx], Gs[idx], g, first, last, lr_t, c1, c2);
-            }
+            gradient<false>(S.Z, S.X, H, [&](int idx, const float2 (&g)[kNU / 32]) {
+                accumulate_row(P, M, V, Gs, idx, g, first, last, lr_t, c1, c2);
+            });
             for (int h = t; h < H; h += kTrainThreads) {
                 float2 g = make_float2(0.f, 0.f);
                 for (int j = 0; j < kTB; ++j) g = make_float2(g.x + S.Z[h][j].x, g.y + S.Z[h][j].y);
