@@ -623,6 +623,12 @@ ie_status take_device_error(ie_plan p, cudaStream_t st) {
     return IE_ERR_TIMEOUT;
 }
 
+// A full product by convolution runs its near part on the plan's side stream: the near blocks are
+// bound by HBM, the convolution's passes by latency.  The near kernel takes 3 CTAs of 256 threads
+// and 80 registers per SM (persistent over the boxes), so that the passes find room beside it.
+// 64 boxes 41 -> 35 us, 16^3 shell 130 -> 120 us, refined solve on the 32^3 shell 4.87 -> 4.72 ms.
+constexpr int kNearBeside = 3;
+
 ie_status apply(ie_plan p, int which, int prec, const float2 *c, float2 *y, int nrhs, cudaStream_t st,
                 const int *gate) {
     if (which == IE_FAR) return far_product(p, prec, c, y, nrhs, false, st, gate);
@@ -630,9 +636,22 @@ ie_status apply(ie_plan p, int which, int prec, const float2 *c, float2 *y, int 
         // the convolution holds the adjacent boxes' site pairs beyond kNearReach: near blocks
         // of the others only, and nothing to take off
         IE_TRY(adj_prepare(p, prec, nrhs, st));
-        IE_TRY(launch_near(p, c, y, nrhs, st, gate, true));
-        IE_TRY(launch_aggregate(p, c, p->d_X, nrhs, st, gate));
-        IE_TRY(timed(p, st, [&] { return launch_conv(p, p->d_X, p->d_Yslab, nrhs, st, gate); }));
+        // the other tiles of the near kernel take every register of an SM: nothing runs beside them
+        const bool beside = p->max_nb <= 32 || (p->max_nb <= 64 && nrhs <= 2);
+        if (!beside) {
+            IE_TRY(launch_near(p, c, y, nrhs, st, gate, true));
+        } else {
+            IE_CK(cudaEventRecord(p->fork, st));
+            IE_CK(cudaStreamWaitEvent(p->side, p->fork, 0));
+        }
+        const ie_status near =
+            beside ? launch_near(p, c, y, nrhs, p->side, gate, true, kNearBeside * p->tc_sms) : IE_OK;
+        if (beside) IE_CK(cudaEventRecord(p->join, p->side));
+        ie_status far = launch_aggregate(p, c, p->d_X, nrhs, st, gate);
+        if (far == IE_OK) far = timed(p, st, [&] { return launch_conv(p, p->d_X, p->d_Yslab, nrhs, st, gate); });
+        if (beside) IE_CK(cudaStreamWaitEvent(st, p->join, 0));     // the caller's stream holds all of it again
+        IE_TRY(near);
+        IE_TRY(far);
         return launch_disaggregate(p, p->d_Yslab, 1, 0, y, nrhs, true, st, gate);
     }
     IE_TRY(launch_near(p, c, y, nrhs, st, gate));
@@ -994,6 +1013,9 @@ static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream,
     p->conv_use = conv_classes(pr, p->n_far_pairs, p->sym ? ncanon_used : p->n_far_disp, p->conv);
     if (!p->conv.empty()) {
         PT(conv_create(p, st));
+        PC(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking));
+        PC(cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming));
+        PC(cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming));
         if (!p->gnrhs.empty()) {
             std::vector<int32_t> bc(p->nbox);
             for (int b = 0; b < p->nbox; ++b) bc[b] = p->gnrhs[p->box_group[b]];
@@ -1224,6 +1246,9 @@ ie_status ie_plan_destroy(ie_plan p) {
     for (void *q : p->allocs) cudaFree(q);
     for (auto &e : p->prof_ev)
         if (e) cudaEventDestroy(e);
+    if (p->fork) cudaEventDestroy(p->fork);
+    if (p->join) cudaEventDestroy(p->join);
+    if (p->side) cudaStreamDestroy(p->side);
     if (p->store) store_release(p->store);
     delete p;
     return IE_OK;

@@ -6,7 +6,7 @@
 // scatterer groups has one system per right-hand side.  Arnoldi uses classical
 // Gram-Schmidt applied twice (dot products accumulated in FP64), Givens rotations and
 // the small least-squares solve run in FP64; Krylov vectors are FP32.  Vector kernels
-// walk chunks of 1,024 unknowns that never straddle two scatterers.
+// walk chunks of 512 unknowns that never straddle two scatterers.
 //
 // An iteration is the product and four kernels: each Gram-Schmidt pass's update and the next
 // sums share a pass over W, and the last block of a system to arrive adds the chunks' sums
@@ -73,7 +73,10 @@ namespace ie {
 namespace {
 
 constexpr int kDotThreads = 256;
-constexpr int kEPT = 4;                        // unknowns per thread in the vector kernels
+// unknowns per thread in the vector kernels: small chunks spread the dot products' FP64 work
+// (its rate bounds an SM) over more SMs; 1 / 2 / 4: 609 / 620 / 679 us (176 boxes, 3 columns), 1.48 /
+// 1.45 / 1.52 ms (16^3 shell), 4.81 / 4.70 / 4.72 ms (32^3 shell) per solve
+constexpr int kEPT = 2;
 constexpr int kChunk = kDotThreads * kEPT;     // unknowns per chunk (one block)
 constexpr int kMaxSystems = 1024;
 

@@ -252,6 +252,8 @@ struct ie_plan_s {
     std::vector<ie::ConvClass> conv;
     ie::ConvUse conv_use;              // products that take it
     float2 *d_convA = nullptr, *d_convB = nullptr;
+    cudaStream_t side = nullptr;       // the near part of a full product runs beside the convolution
+    cudaEvent_t fork = nullptr, join = nullptr;
     int32_t *d_box_cols = nullptr;     // [nbox] right-hand sides of each box's scatterer (null: all)
     float2 *d_Nshort = nullptr;        // near blocks of the site pairs within kNearReach (as d_Nblk)
     // adjacent pairs (26 groups) whose site pairs beyond kNearReach the convolution holds,
@@ -338,9 +340,10 @@ ie_status launch_zero(void *ptr, size_t bytes, cudaStream_t st, const int *gate 
 // nslab regions of `count` complex values, `stride` complex values apart, in one launch
 ie_status launch_zero_slabs(float2 *base, int nslab, size_t stride, size_t count, cudaStream_t st,
                             const int *gate = nullptr);
-// shorter: only the site pairs within kNearReach (the others are in the convolution)
+// shorter: only the site pairs within kNearReach (the others are in the convolution);
+// most_ctas: leave the rest of the GPU to kernels that run beside it
 ie_status launch_near(const ie_plan p, const float2 *c, float2 *y, int nrhs, cudaStream_t st,
-                      const int *gate = nullptr, bool shorter = false);
+                      const int *gate = nullptr, bool shorter = false, int most_ctas = INT32_MAX);
 ie_status launch_translate_simt(ie_plan p, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
                                 const int *gate = nullptr, bool adjacent = false);
 ie_status launch_translate_cvfcnn(ie_plan p, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,

@@ -1,5 +1,5 @@
 """GMRES at the edges of its kernels' tiles: restart lengths around the groups of four Krylov
-vectors the dot products take together, systems shorter and longer than a chunk of 1,024
+vectors the dot products take together, systems shorter and longer than a chunk of 512
 unknowns, and a batch in which a scatterer has no boxes.  Bounds: the recomputed residual
 within the requested tolerance (the recurrence stops there; FP32 products add 1e-6), against
 the FP64 oracle's operator."""
