@@ -207,6 +207,7 @@ constexpr int x_line() { return R1 * (R2 + 1) + 5; }
 
 template <int R1, int R2>
 __global__ void __launch_bounds__(kXThreads) conv_x_kernel(const ConvArgs a) {
+    chain_wait();
     if (a.gate && *a.gate == 0) return;
     constexpr int L = R1 * R2, rows = XTile<R2>::rows, LS = x_line<R1, R2>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(kXThreads) conv_x_kernel(const ConvArgs a) {
             v[i] = make_float2(0.f, 0.f);
             if (y < ny && n < nx) {
                 const int box = __ldg(sl + (n >> 2));
-                if (box >= 0) v[i] = __ldg(x + (int64_t)box * kNU + 3 * (n & 3));
+                if (box >= 0) v[i] = x[(int64_t)box * kNU + 3 * (n & 3)];
             }
         });
         dft_half_in<R1>(v);
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(kXThreads) conv_x_kernel(const ConvArgs a) {
 
 template <int R1, int R2>
 __global__ void __launch_bounds__(kXThreads) conv_xback_kernel(const ConvArgs a) {
+    chain_wait();
     if (a.gate && *a.gate == 0) return;
     constexpr int L = R1 * R2, rows = XTile<R2>::rows, LS = x_line<R1, R2>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -299,6 +301,7 @@ __global__ void __launch_bounds__(kXThreads) conv_xback_kernel(const ConvArgs a)
 // y pass of one (component, plane z, kx tile)
 template <int R1, int R2>
 __global__ void __launch_bounds__(kW *R2) conv_y_kernel(const ConvArgs a) {
+    chain_wait();
     if (a.gate && *a.gate == 0) return;
     constexpr int L = R1 * R2, NT = kW * R2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -332,6 +335,7 @@ __global__ void __launch_bounds__(kW *R2) conv_y_kernel(const ConvArgs a) {
 
 template <int R1, int R2>
 __global__ void __launch_bounds__(kW *R2) conv_yback_kernel(const ConvArgs a) {
+    chain_wait();
     if (a.gate && *a.gate == 0) return;
     constexpr int L = R1 * R2, NT = kW * R2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -382,6 +386,7 @@ __device__ __forceinline__ void cmac(float2 &d, float2 a, float2 b) {
 // PFMAX: points of K^ fetched ahead of their use; AHEAD: the three components' lines too.
 template <int R1, int R2, int PFMAX, bool AHEAD, int CTAS>
 __global__ void __launch_bounds__(kW *R2, CTAS) conv_z_kernel(const ConvArgs a) {
+    chain_wait();
     if (a.gate && *a.gate == 0) return;
     constexpr int L = R1 * R2, NT = kW * R2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -807,7 +812,17 @@ int64_t conv_traffic(const ie_plan_s *p, int nrhs) {
     return b;
 }
 
+// The passes of a small convolution take 3 to 30 us each, and a launch's set-up and ramp about 1.5
+// us: they are chained (launch_after).  64 boxes (L = 32) 35 -> 28 us, 16^3 shell (L = 128) 126 ->
+// 116, 8 scatterers with four columns 1,099 -> 1,060.  Not from L = 256 on (32^3 shell far 571 ->
+// 577 us: the next pass's CTAs hold room beside a long pass) and not under capture (as edges of the
+// GMRES cycle's graph: 16^3 shell solve 1,510 -> 1,522 us, 32^3 shell 4,731 -> 4,901).
+constexpr int64_t kEarlyPoints = (int64_t)192 * 192 * 192;
+
 ie_status launch_conv(ie_plan p, const float2 *X, float2 *Y, int nrhs, cudaStream_t st, const int *gate) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    IE_CK(cudaStreamIsCapturing(st, &cs));
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
     for (const auto &c : p->conv) {
         ConvArgs a;
         a.X = X;
@@ -827,33 +842,34 @@ ie_status launch_conv(ie_plan p, const float2 *X, float2 *Y, int nrhs, cudaStrea
         a.nbox = p->nbox;
         a.nrhs = nrhs;
         a.gate = gate;
+        const bool early = !capturing && (int64_t)a.Lx * a.Ly * a.Lz <= kEarlyPoints;
         const int cols = (int)c.group.size() * nrhs, ny = 4 * a.Ey, nz = 4 * a.Ez;
         for (a.q0 = 0; a.q0 < cols; a.q0 += c.chunk) {
             const unsigned nq = (unsigned)std::min(c.chunk, cols - a.q0);
             auto xgrid = [&](int rows) { return dim3((unsigned)((ny + rows - 1) / rows), (unsigned)nz, nq); };
             const dim3 ygrid(a.Lx / kW, nz, 3 * nq), zgrid(a.Lx / kW, a.Ly, nq);
 #define IE_CASE(L, R1, R2) \
-    case L: conv_x_kernel<R1, R2><<<xgrid(XTile<R2>::rows), kXThreads, x_smem<R1, R2>(), st>>>(a); break;
+    case L: launch_after(early, conv_x_kernel<R1, R2>, xgrid(XTile<R2>::rows), kXThreads, x_smem<R1, R2>(), st, a); break;
             switch (a.Lx) { IE_CONV_SIZES(IE_CASE) }
 #undef IE_CASE
             IE_CK_LAUNCH();
 #define IE_CASE(L, R1, R2) \
-    case L: conv_y_kernel<R1, R2><<<ygrid, kW * R2, y_smem<R1, R2>(), st>>>(a); break;
+    case L: launch_after(early, conv_y_kernel<R1, R2>, ygrid, kW * R2, y_smem<R1, R2>(), st, a); break;
             switch (a.Ly) { IE_CONV_SIZES(IE_CASE) }
 #undef IE_CASE
             IE_CK_LAUNCH();
 #define IE_CASE(L, R1, R2, PF, AHEAD, CTAS) \
-    case L: conv_z_kernel<R1, R2, PF, AHEAD, CTAS><<<zgrid, kW * R2, z_smem<R1, R2>(), st>>>(a); break;
+    case L: launch_after(early, conv_z_kernel<R1, R2, PF, AHEAD, CTAS>, zgrid, kW * R2, z_smem<R1, R2>(), st, a); break;
             switch (a.Lz) { IE_CONV_ZSIZES(IE_CASE) }
 #undef IE_CASE
             IE_CK_LAUNCH();
 #define IE_CASE(L, R1, R2) \
-    case L: conv_yback_kernel<R1, R2><<<ygrid, kW * R2, y_smem<R1, R2>(), st>>>(a); break;
+    case L: launch_after(early, conv_yback_kernel<R1, R2>, ygrid, kW * R2, y_smem<R1, R2>(), st, a); break;
             switch (a.Ly) { IE_CONV_SIZES(IE_CASE) }
 #undef IE_CASE
             IE_CK_LAUNCH();
 #define IE_CASE(L, R1, R2) \
-    case L: conv_xback_kernel<R1, R2><<<xgrid(XTile<R2>::rows), kXThreads, x_smem<R1, R2>(), st>>>(a); break;
+    case L: launch_after(early, conv_xback_kernel<R1, R2>, xgrid(XTile<R2>::rows), kXThreads, x_smem<R1, R2>(), st, a); break;
             switch (a.Lx) { IE_CONV_SIZES(IE_CASE) }
 #undef IE_CASE
             IE_CK_LAUNCH();

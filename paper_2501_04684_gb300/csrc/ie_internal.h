@@ -122,6 +122,30 @@ void capture_end();
         }                                                                              \
     } while (0)
 
+// Chains of short kernels: a kernel launched by launch_after with `early` may be set up and take
+// its place on the SMs while the one before it on the stream drains (programmatic stream
+// serialisation).  It starts with chain_wait(), which returns when everything before it has
+// finished and is visible, so nothing it reads may come from earlier kernels through the
+// read-only path (__ldg, const __restrict__) and it touches nothing before the wait.
+// chain_next() lets the follower in.
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_next() { cudaTriggerProgrammaticLaunchCompletion(); }
+__device__ __forceinline__ void chain_wait() {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+}
+#endif
+template <class... P, class... A>
+void launch_after(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid, c.blockDim = block, c.dynamicSmemBytes = smem, c.stream = st;
+    c.attrs = &at, c.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, P(args)...);     // IE_CK_LAUNCH reads its error
+}
+
 #define IE_TRY(expr)                                                                   \
     do {                                                                               \
         ie_status s_ = (expr);                                                         \

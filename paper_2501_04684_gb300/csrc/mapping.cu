@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(kNU) aggregate_kernel(const float2 *__restrict
                                                         const int64_t *__restrict__ off, int64_t n, int nbox,
                                                         const float2 *__restrict__ c, float2 *__restrict__ X, int nrhs,
                                                         const int *__restrict__ gate) {
+    chain_next();
     if (gate && *gate == 0) return;
     __shared__ float2 cs[kNU + 16][NR];
     const int b = blockIdx.x, r0 = blockIdx.y * NR, u = threadIdx.x;
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(kDisThreads) disaggregate_kernel(const float2 
                                                            const float2 *__restrict__ Yslab, int nslab,
                                                            size_t slab_stride, float2 *__restrict__ out, int accumulate,
                                                            int identity, int nrhs, const int *__restrict__ gate) {
+    chain_next();
     if (gate && *gate == 0) return;
     constexpr int kRows = 4, M = 2 * kRows * NR;
     __shared__ float2 ys[NR][kNU];
