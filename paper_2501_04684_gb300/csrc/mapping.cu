@@ -67,33 +67,35 @@ __global__ void copy_kernel(const float4 *__restrict__ a, float4 *__restrict__ b
 }
 
 // 16-bit hi/lo split of X for the tensor-core path.  Layout [hl][rhs][nbox][chunk][reim][32]:
-// per column 384 values, K-chunk major (chunk = u / 32), re and im rows of a chunk adjacent.
+// per column 384 values, K-chunk major (chunk = u / 32), re and im rows of a chunk adjacent, so
+// one K-chunk of a column (both rows) is 128 contiguous bytes for the tensor-core gathers.
 // FP16: the column is scaled by 2^-e so that max |x| < 2^14; e is stored.
-// With a symmetry map, block z writes copy z of the signed-permuted input
-// x^Q[u] = +-x[U_Q(u)] at Xtc + z * (2 planes); the scale is the same for every copy.
+// With a symmetry map, copy z holds the signed-permuted input x^Q[u] = +-x[U_Q(u)] at Xtc + z *
+// (2 planes); the scale is the same for every copy.
+//
+// Bound by the writes (48 copies: 74 KB per column).  A CTA splits its column once, keeps the
+// halves in shared memory and writes kSplitCopies copies with 16-byte stores: a thread gathers
+// eight unknowns of one copy and writes their four lines (hi, lo of re, im).  920 boxes, 48
+// copies: network product 763 -> 739 us (a CTA per copy with 2-byte stores took 43 us of it).
+constexpr int kSplitCopies = 8;
+static_assert(kNU / 8 * kSplitCopies == kNU, "one thread per eight unknowns of a copy");
+static_assert(kSym % kSplitCopies == 0, "whole groups of copies");
 template <bool FP16>
-__global__ void split_kernel(const float2 *__restrict__ X, int nbox, int nrhs, uint16_t *__restrict__ Xtc,
-                             int32_t *__restrict__ Xexp, float *__restrict__ Xinf, const uint16_t *__restrict__ symmap,
-                             const int *__restrict__ gate) {
+__global__ void __launch_bounds__(kNU)
+split_kernel(const float2 *__restrict__ X, int nbox, int nrhs, uint16_t *__restrict__ Xtc, int32_t *__restrict__ Xexp,
+             float *__restrict__ Xinf, const uint16_t *__restrict__ symmap, const int *__restrict__ gate) {
     if (gate && *gate == 0) return;
-    int b = blockIdx.x, r = blockIdx.y, u = threadIdx.x;
-    const int sg = blockIdx.z;
-    int64_t col = (int64_t)r * nbox + b;
-    float2 x;
-    if (symmap) {
-        const uint16_t e = symmap[sg * kNU + u];
-        x = X[col * kNU + (e & 0xFF)];
-        if (e & 0x100) x = make_float2(-x.x, -x.y);
-    } else {
-        x = X[col * kNU + u];
-    }
-    const bool write_exp = sg == 0;
+    __shared__ uint2 halves[kNU];           // (hi re, hi im), (lo re, lo im)
+    const int b = blockIdx.x, r = blockIdx.y, u = threadIdx.x;
+    const int64_t col = (int64_t)r * nbox + b;
+    const float2 x = X[col * kNU + u];
+    const bool write_exp = blockIdx.z == 0;
     float scale = 1.f;
     if (FP16) {
         __shared__ float red[8], red2[8];
         __shared__ float s_scale;
         float m = fmaxf(fabsf(x.x), fabsf(x.y));
-        float m2 = x.x * x.x + x.y * x.y;     // for max_u |x_u| (the networks' input norm)
+        float m2 = fmaf(x.y, x.y, x.x * x.x);     // for max_u |x_u| (the networks' input norm)
         for (int o = 16; o; o >>= 1) {
             m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
             m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, o));
@@ -117,12 +119,8 @@ __global__ void split_kernel(const float2 *__restrict__ X, int nbox, int nrhs, u
     } else if (u == 0 && write_exp) {
         Xexp[col] = 0;
     }
-    int64_t plane = (int64_t)nrhs * nbox * 2 * kNU;
-    // K-chunk-major within the column: [chunk of 32][re 32, im 32], so one K-chunk of a
-    // column (both rows) is 128 contiguous bytes for the tensor-core gathers
-    uint16_t *cre = Xtc + 2 * plane * sg + (col * 2) * kNU + (u >> 5) * 64 + (u & 31);
-    float v[2] = {x.x * scale, x.y * scale};
-    uint16_t hi[2], lo[2];
+    const float v[2] = {x.x * scale, x.y * scale};
+    uint32_t hi[2], lo[2];
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
         if (FP16) {
@@ -135,10 +133,59 @@ __global__ void split_kernel(const float2 *__restrict__ X, int nbox, int nrhs, u
             lo[t] = __bfloat16_as_ushort(__float2bfloat16_rn(v[t] - __bfloat162float(h)));
         }
     }
-    cre[0] = hi[0];
-    cre[32] = hi[1];
-    cre[plane] = lo[0];
-    cre[plane + 32] = lo[1];
+    const int64_t plane = (int64_t)nrhs * nbox * 2 * kNU;
+    if (!symmap) {                          // one copy: every thread writes its own unknown
+        uint16_t *cre = Xtc + col * 2 * kNU + (u >> 5) * 64 + (u & 31);
+        cre[0] = hi[0];
+        cre[32] = hi[1];
+        cre[plane] = lo[0];
+        cre[plane + 32] = lo[1];
+        return;
+    }
+    halves[u] = make_uint2(hi[0] | hi[1] << 16, lo[0] | lo[1] << 16);
+    __syncthreads();
+    const int sg = blockIdx.z * kSplitCopies + u / (kNU / 8), k = u % (kNU / 8);    // copy, eight unknowns
+    const uint4 e = __ldg(reinterpret_cast<const uint4 *>(symmap + (size_t)sg * kNU) + k);
+    const uint32_t w[4] = {e.x, e.y, e.z, e.w};
+    uint2 h[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t from = w[i >> 1] >> (16 * (i & 1));
+        h[i] = halves[from & 0xFF];
+        const uint32_t neg = from & 0x100 ? 0x80008000u : 0u;        // the halves of -x are negated
+        h[i].x ^= neg;
+        h[i].y ^= neg;
+    }
+    uint16_t *out = Xtc + 2 * plane * sg + col * 2 * kNU + (k >> 2) * 64 + (k & 3) * 8;
+    uint4 re[2], im[2];                     // hi, lo: low halves of a pair of words are re, high ones im
+    re[0] = make_uint4(__byte_perm(h[0].x, h[1].x, 0x5410), __byte_perm(h[2].x, h[3].x, 0x5410),
+                       __byte_perm(h[4].x, h[5].x, 0x5410), __byte_perm(h[6].x, h[7].x, 0x5410));
+    im[0] = make_uint4(__byte_perm(h[0].x, h[1].x, 0x7632), __byte_perm(h[2].x, h[3].x, 0x7632),
+                       __byte_perm(h[4].x, h[5].x, 0x7632), __byte_perm(h[6].x, h[7].x, 0x7632));
+    re[1] = make_uint4(__byte_perm(h[0].y, h[1].y, 0x5410), __byte_perm(h[2].y, h[3].y, 0x5410),
+                       __byte_perm(h[4].y, h[5].y, 0x5410), __byte_perm(h[6].y, h[7].y, 0x5410));
+    im[1] = make_uint4(__byte_perm(h[0].y, h[1].y, 0x7632), __byte_perm(h[2].y, h[3].y, 0x7632),
+                       __byte_perm(h[4].y, h[5].y, 0x7632), __byte_perm(h[6].y, h[7].y, 0x7632));
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        *reinterpret_cast<uint4 *>(out + t * plane) = re[t];
+        *reinterpret_cast<uint4 *>(out + t * plane + 32) = im[t];
+    }
+}
+
+// Sum of an entry's nslab <= kSlabs partial sums (FP64), their reads in flight together (eight slabs
+// added in a loop cost the inverse mapping of 920 boxes 24 us).
+__device__ __forceinline__ float2 slab_sum(const float2 *__restrict__ Y, int nslab, size_t slab_stride) {
+    float2 w[kSlabs];
+#pragma unroll
+    for (int s = 0; s < kSlabs; ++s) w[s] = s < nslab ? Y[s * slab_stride] : make_float2(0.f, 0.f);
+    double sr = 0, si = 0;
+#pragma unroll
+    for (int s = 0; s < kSlabs; ++s) {
+        sr += w[s].x;
+        si += w[s].y;
+    }
+    return make_float2((float)sr, (float)si);
 }
 
 // r[i] (+)= sum_u P[i][u] y[u], y = sum over slabs (FP64), for NR right-hand sides (P is read
@@ -167,14 +214,12 @@ __global__ void __launch_bounds__(kDisThreads) disaggregate_kernel(const float2 
             const float2 *Y = Yslab + ((int64_t)(r0 + r) * nbox + b) * kNU + u;
             if (nslab == 1) {
                 v = *Y;
+            } else if (nslab == 2) {
+                v = *Y;
+                const float2 w = Y[slab_stride];
+                v = make_float2((float)((double)v.x + w.x), (float)((double)v.y + w.y));
             } else {
-                double sr = 0, si = 0;
-                for (int s = 0; s < nslab; ++s) {
-                    const float2 w = Y[s * slab_stride];
-                    sr += w.x;
-                    si += w.y;
-                }
-                v = make_float2((float)sr, (float)si);
+                v = slab_sum(Y, nslab, slab_stride);
             }
         }
         ys[r][u] = v;
@@ -266,13 +311,7 @@ __global__ void sum_slabs_kernel(const float2 *__restrict__ Yslab, int nslab, si
                                  float2 *__restrict__ Y) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
-    double sr = 0, si = 0;
-    for (int s = 0; s < nslab; ++s) {
-        float2 v = Yslab[s * slab_stride + i];
-        sr += v.x;
-        si += v.y;
-    }
-    Y[i] = make_float2((float)sr, (float)si);
+    Y[i] = slab_sum(Yslab + i, nslab, slab_stride);
 }
 
 // Plane wave at the dipole sites, e[3s+a] = pol[a] exp(-j k khat . r_s) (FP64 phase),
@@ -350,7 +389,7 @@ ie_status launch_aggregate(const ie_plan p, const float2 *c, float2 *X, int nrhs
 ie_status launch_split_tc(const ie_plan p, const float2 *X, int nrhs, bool fp16, cudaStream_t st, const int *gate,
                           bool plain) {
     const bool sym = p->sym && !plain;
-    const dim3 grid(p->nbox, nrhs, sym ? kSym : 1);
+    const dim3 grid(p->nbox, nrhs, sym ? kSym / kSplitCopies : 1);
     const uint16_t *map = sym ? p->d_symmap : nullptr;
     if (fp16)
         split_kernel<true><<<grid, kNU, 0, st>>>(X, p->nbox, nrhs, p->d_Xtc, p->d_Xexp, p->d_Xinf, map, gate);
