@@ -173,8 +173,7 @@ split_kernel(const float2 *__restrict__ X, int nbox, int nrhs, uint16_t *__restr
     }
 }
 
-// Sum of an entry's nslab <= kSlabs partial sums (FP64), their reads in flight together (eight slabs
-// added in a loop cost the inverse mapping of 920 boxes 24 us).
+// Sum of an entry's nslab <= kSlabs partial sums (FP64), their reads in flight together.
 __device__ __forceinline__ float2 slab_sum(const float2 *__restrict__ Y, int nslab, size_t slab_stride) {
     float2 w[kSlabs];
 #pragma unroll
