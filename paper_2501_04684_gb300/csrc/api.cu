@@ -393,6 +393,29 @@ size_t plan_bytes(const ie_problem *pr, int64_t n, int64_t npairs, int64_t nd, i
     return b;
 }
 
+// Device copy of a work list, made in the first call that needs it: also while the caller's
+// stream is being captured (the list is then no part of the graph; a private stream copies it).
+ie_status upload_list(ie_plan p, const std::vector<WorkItem> &items, WorkList &wl) {
+    wl.n = (int64_t)items.size();
+    if (!wl.n) return IE_OK;
+    const size_t bytes = items.size() * sizeof(WorkItem);
+    std::lock_guard<std::recursive_mutex> lock(device_mutex());
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    IE_CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    cudaStream_t own = nullptr;
+    auto body = [&]() -> ie_status {
+        IE_TRY(dalloc_t(p, &wl.d_items, items.size()));
+        IE_CK(cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking));
+        IE_CK(cudaMemcpyAsync(wl.d_items, items.data(), bytes, cudaMemcpyHostToDevice, own));
+        IE_CK(cudaStreamSynchronize(own));
+        return IE_OK;
+    };
+    const ie_status rc = body();
+    if (own) cudaStreamDestroy(own);
+    IE_CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    return rc;
+}
+
 }  // namespace
 
 // Work list of one translation kernel for `nrhs`: every displacement group cut into
@@ -456,11 +479,7 @@ ie_status work_list(ie_plan p, bool tc, int nrhs, WorkList **out, int max_cols, 
         std::stable_sort(items.begin(), items.end(),
                          [](const WorkItem &a, const WorkItem &b) { return a.npairs * a.nr > b.npairs * b.nr; });
     WorkList wl;
-    wl.n = (int64_t)items.size();
-    if (wl.n) {
-        IE_TRY(dalloc_t(p, &wl.d_items, items.size()));
-        IE_CK(cudaMemcpy(wl.d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
-    }
+    IE_TRY(upload_list(p, items, wl));
     if (tc)
         p->n_work_tc = wl.n;
     else
@@ -554,25 +573,10 @@ ie_status adj_list(ie_plan p, bool tc, int nrhs, WorkList **out) {
             q += np;
         }
     WorkList wl;
-    wl.n = (int64_t)items.size();
-    if (wl.n) {
-        IE_TRY(dalloc_t(p, &wl.d_items, items.size()));
-        IE_CK(cudaMemcpy(wl.d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
-    }
+    IE_TRY(upload_list(p, items, wl));
     p->adj_work[key] = wl;
     *out = &p->adj_work[key];
     return IE_OK;
-}
-
-// Makes the list a far product of this nrhs will want (outside any capture), as a full
-// product with block products would have made the list they share.
-static ie_status adj_prepare(ie_plan p, int prec, int nrhs, cudaStream_t st) {
-    const bool tc = prec != IE_PREC_FP32;
-    if (!p->n_adj || p->adj_work.count(2 * nrhs + (tc ? 1 : 0))) return IE_OK;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    IE_CK(cudaStreamIsCapturing(st, &cs));
-    WorkList *wl = nullptr;
-    return cs == cudaStreamCaptureStatusNone ? adj_list(p, tc, nrhs, &wl) : IE_OK;
 }
 
 ie_status launch_adjacent(ie_plan p, int prec, const float2 *X, float2 *slab, int nrhs, cudaStream_t st,
@@ -635,7 +639,6 @@ ie_status apply(ie_plan p, int which, int prec, const float2 *c, float2 *y, int 
     if (which == IE_FULL && conv_full(p, prec)) {
         // the convolution holds the adjacent boxes' site pairs beyond kNearReach: near blocks
         // of the others only, and nothing to take off
-        IE_TRY(adj_prepare(p, prec, nrhs, st));
         // the other tiles of the near kernel take every register of an SM: nothing runs beside them
         const bool beside = p->max_nb <= 32 || (p->max_nb <= 64 && nrhs <= 2);
         if (!beside) {
