@@ -89,12 +89,20 @@ typedef enum {
  *  CVFCNN_FP32  the same networks evaluated in FP32 on the SIMT cores. */
 /*
  * Evaluation: all boxes' dipoles lie on one lattice, so the far field is a discrete
- * convolution of D (eq. 5).  Products in FP32, BF16X3 and FP16X3 are evaluated as such in
- * FP32 (its error against FP64 is below that of the block products in these precisions)
- * where the scatterers' bounding lattices make it the cheaper form and k a >= 0.75; the
- * products of the adjacent boxes' site pairs that it holds besides are taken off in the named
- * arithmetic, or left to it (IE_FULL).  Otherwise, and in the other precisions always, the
- * block products per displacement run in the named arithmetic. */
+ * convolution of D (eq. 5).  Where the scatterers' bounding lattices make that the cheaper
+ * form and k a >= 0.75, products in FP32, BF16X3 and FP16X3 are evaluated as one, in FP32.
+ * Its rounding is relative to the scatterer's whole field, that of a block product to what
+ * reaches the box:
+ *  - IE_FULL products (and solves): the near part holds the boxes where that would matter;
+ *    measured box by box, the error against FP64 is that of the FP32 block products.
+ *  - IE_FAR and ie_translate: the adjacent boxes' site pairs that the convolution holds
+ *    besides are taken off in the named arithmetic.  It serves the calls in which, for every
+ *    box and column, the far boxes hold at least a quarter of the scatterer's sum |x_u|^2 (a
+ *    box's error is then at most about twice the FP32 block products').  Calls with other
+ *    inputs (strong contrasts, a lone source, NaN or infinite values) are decided on the
+ *    device and take the block products.
+ * Otherwise, and in the other precisions always, the block products per displacement run in
+ * the named arithmetic. */
 typedef enum {
     IE_PREC_FP32 = 1,
     IE_PREC_BF16X3 = 2,

@@ -326,10 +326,11 @@ void near_lists(const ie_problem *pr, const BoxGrid &g, const std::vector<int32_
     start[n] = (int32_t)src.size();
 }
 
-size_t plan_bytes(const ie_problem *pr, int64_t n, int64_t npairs, int64_t nd, int64_t nnear, int64_t near_elems,
-                  int64_t nblk, bool shared = false, int64_t used = -1) {
+size_t plan_bytes(const ie_problem *pr, int64_t n, int64_t npairs, int64_t nd, const std::vector<int32_t> &near_start,
+                  int64_t near_elems, int64_t nblk, bool shared = false, int64_t used = -1) {
+    const int64_t nnear = near_start.back();
     std::vector<ConvClass> conv;      // used: stored blocks the pairs use (a shared store holds more)
-    const ConvUse use = conv_classes(pr, npairs, used >= 0 ? used : pr->symmetry == 1 ? nblk : nd, conv);
+    const ConvUse use = conv_classes(pr, npairs, used >= 0 ? used : pr->symmetry == 1 ? nblk : nd, near_start, conv);
     size_t b = conv_bytes(pr, conv, use, nnear, near_elems);
     auto add = [&](size_t x) { b += (x + 255) / 256 * 256; };
     int64_t nbox = pr->n_boxes;
@@ -541,16 +542,6 @@ static ie_status timed(ie_plan p, cudaStream_t st, F body) {
     return IE_OK;
 }
 
-ie_status translate_timed(ie_plan p, int prec, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
-                          const int *gate) {
-    return timed(p, st, [&] {
-        if (prec == IE_PREC_FP32) return launch_translate_simt(p, X, Yslab, nrhs, st, gate);
-        if (prec == IE_PREC_CVFCNN_FP32) return launch_translate_cvfcnn(p, X, Yslab, nrhs, st, gate);
-        if (prec == IE_PREC_CVFCNN) return launch_translate_cvfcnn_tc(p, Yslab, nrhs, st, gate);
-        return launch_translate_tc(p, prec, Yslab, nrhs, st, gate);
-    });
-}
-
 // Work list of the adjacent pairs (launch_adjacent): runs of one displacement's pairs.
 ie_status adj_list(ie_plan p, bool tc, int nrhs, WorkList **out) {
     const int key = 2 * nrhs + (tc ? 1 : 0), cols = tc ? tc_tile_columns() : simt_tile_columns();
@@ -588,33 +579,65 @@ ie_status launch_adjacent(ie_plan p, int prec, const float2 *X, float2 *slab, in
 
 // The far field of X by convolution in two slabs of the scratch: the adjacent pairs'
 // (negated) part of it, and the convolution itself.
-static ie_status conv_translate(ie_plan p, int prec, const float2 *X, int nrhs, int *nslab, cudaStream_t st,
-                                const int *gate) {
+static ie_status conv_translate(ie_plan p, int prec, const float2 *X, int nrhs, cudaStream_t st, const int *gate) {
     const size_t stride = slab_stride(p);
-    *nslab = 1;
     float2 *Y = p->d_Yslab;
     if (p->n_adj) {
         IE_TRY(launch_zero_slabs(p->d_Yslab, 1, stride, (size_t)nrhs * p->nbox * kNU, st, gate));
         IE_TRY(launch_adjacent(p, prec, X, p->d_Yslab, nrhs, st, gate));
         Y += stride;
-        *nslab = 2;
     }
     return launch_conv(p, X, Y, nrhs, st, gate);
 }
 
+// Its block products.
+static ie_status block_translate(ie_plan p, int prec, const float2 *X, int nrhs, cudaStream_t st, const int *gate,
+                                 int most_ctas = INT32_MAX) {
+    IE_TRY(launch_zero_slabs(p->d_Yslab, kSlabs, slab_stride(p), (size_t)nrhs * p->nbox * kNU, st, gate, most_ctas));
+    if (uses_split(prec)) IE_TRY(launch_split_tc(p, X, nrhs, is_fp16(prec), st, gate, false, most_ctas));
+    return timed(p, st, [&] {
+        if (prec == IE_PREC_FP32) return launch_translate_simt(p, X, p->d_Yslab, nrhs, st, gate, false, most_ctas);
+        if (prec == IE_PREC_CVFCNN_FP32) return launch_translate_cvfcnn(p, X, p->d_Yslab, nrhs, st, gate);
+        if (prec == IE_PREC_CVFCNN) return launch_translate_cvfcnn_tc(p, p->d_Yslab, nrhs, st, gate);
+        return launch_translate_tc(p, prec, p->d_Yslab, nrhs, st, gate);
+    });
+}
+
+// The far field of X in the form its values call for (kFarEven), which sum(slabs, form) takes from
+// the scratch.  The convolution always runs, and the side stream looks at the values meanwhile;
+// the blocks follow, gated by what it found, in few CTAs: 32^3 shell (FP16X3) 589 us with
+// even inputs, 566 without the choice; 599 with the choice first, the blocks beside the convolution
+// and a gate to read in every kernel.
+template <class Sum>
+static ie_status chosen_translate(ie_plan p, int prec, const float2 *X, int nrhs, cudaStream_t st, const int *gate,
+                                  Sum sum) {
+    IE_TRY(timed(p, st, [&] {
+        IE_CK(cudaEventRecord(p->fork, st));
+        IE_CK(cudaStreamWaitEvent(p->side, p->fork, 0));
+        const ie_status form = launch_choose_form(p, X, nrhs, p->side, gate);
+        IE_CK(cudaEventRecord(p->join, p->side));
+        const ie_status conv = conv_translate(p, prec, X, nrhs, st, gate);
+        IE_CK(cudaStreamWaitEvent(st, p->join, 0));
+        IE_TRY(form);
+        IE_TRY(conv);
+        const int profile = p->profile;
+        p->profile = 0;                             // the bracket is this one
+        const ie_status blocks = block_translate(p, prec, X, nrhs, st, p->d_form + 1, 2 * p->tc_sms);
+        p->profile = profile;
+        return blocks;
+    }));
+    return sum(p->n_adj ? 2 : 1, p->d_form);
+}
+
 ie_status far_product(ie_plan p, int prec, const float2 *c, float2 *y, int nrhs, bool accumulate, cudaStream_t st,
                       const int *gate) {
-    size_t stride = slab_stride(p);
     IE_TRY(launch_aggregate(p, c, p->d_X, nrhs, st, gate));
-    int nslab = kSlabs;
-    if (conv_far(p, prec)) {
-        IE_TRY(timed(p, st, [&] { return conv_translate(p, prec, p->d_X, nrhs, &nslab, st, gate); }));
-    } else {
-        IE_TRY(launch_zero_slabs(p->d_Yslab, kSlabs, stride, (size_t)nrhs * p->nbox * kNU, st, gate));
-        if (uses_split(prec)) IE_TRY(launch_split_tc(p, p->d_X, nrhs, is_fp16(prec), st, gate));
-        IE_TRY(translate_timed(p, prec, p->d_X, p->d_Yslab, nrhs, st, gate));
-    }
-    return launch_disaggregate(p, p->d_Yslab, nslab, stride, y, nrhs, accumulate, st, gate);
+    auto map_back = [&](int nslab, const int *form) {
+        return launch_disaggregate(p, p->d_Yslab, nslab, slab_stride(p), y, nrhs, accumulate, st, gate, form);
+    };
+    if (conv_far(p, prec)) return chosen_translate(p, prec, p->d_X, nrhs, st, gate, map_back);
+    IE_TRY(block_translate(p, prec, p->d_X, nrhs, st, gate));
+    return map_back(kSlabs, nullptr);
 }
 
 ie_status take_device_error(ie_plan p, cudaStream_t st) {
@@ -713,7 +736,7 @@ ie_status ie_plan_footprint(const ie_problem *pr, size_t *bytes) {
     std::vector<int64_t> boff;
     int64_t elems = 0;
     near_lists(pr, g, nb, st, src, boff, elems);
-    *bytes = plan_bytes(pr, n, npairs, nd, (int64_t)src.size(), elems, ncanon);
+    *bytes = plan_bytes(pr, n, npairs, nd, st, elems, ncanon);
     return IE_OK;
 }
 
@@ -1013,7 +1036,7 @@ static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream,
     }
 
     // far product as a convolution: its blocks of the adjacent pairs, K^, workspace
-    p->conv_use = conv_classes(pr, p->n_far_pairs, p->sym ? ncanon_used : p->n_far_disp, p->conv);
+    p->conv_use = conv_classes(pr, p->n_far_pairs, p->sym ? ncanon_used : p->n_far_disp, nstart, p->conv);
     if (!p->conv.empty()) {
         PT(conv_create(p, st));
         PC(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking));
@@ -1026,6 +1049,11 @@ static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream,
             PC(cudaMemcpy(p->d_box_cols, bc.data(), bc.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
         }
         if (p->conv_use.far) {
+            const std::vector<int32_t> gb(p->gbox.begin(), p->gbox.end());
+            PT(dalloc_t(p, &p->d_gbox, gb.size()));
+            PT(dalloc_t(p, &p->d_energy, (size_t)p->max_rhs * p->nbox));
+            PT(dalloc_t(p, &p->d_form, 2));
+            PC(cudaMemcpy(p->d_gbox, gb.data(), gb.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
             std::vector<int32_t> asrc, adst;
             p->h_adj_start.assign(28, 0);
             for (int e = 0; e < 27; ++e) {
@@ -1125,7 +1153,7 @@ ie_status ie_plan_footprint_shared(const ie_problem *pr, ie_store store, size_t 
     std::vector<int64_t> boff;
     int64_t elems = 0;
     near_lists(pr, g, nb, st, src, boff, elems);
-    *bytes = plan_bytes(pr, n, npairs, nd, (int64_t)src.size(), elems, store->n_blocks, true, ncanon);
+    *bytes = plan_bytes(pr, n, npairs, nd, st, elems, store->n_blocks, true, ncanon);
     return IE_OK;
 }
 
@@ -1279,16 +1307,12 @@ ie_status ie_translate(ie_plan p, int prec, const void *X, void *Y, int nrhs, vo
     IE_TRY(check_rhs(p, nrhs));
     IE_TRY(check_prec(p, prec));
     cudaStream_t st = (cudaStream_t)stream;
-    size_t stride = slab_stride(p);
-    if (conv_far(p, prec)) {
-        int nslab = 0;
-        IE_TRY(timed(p, st, [&] { return conv_translate(p, prec, (const float2 *)X, nrhs, &nslab, st, nullptr); }));
-        return launch_sum_slabs(p, p->d_Yslab, nslab, stride, (float2 *)Y, nrhs, st);
-    }
-    IE_TRY(launch_zero_slabs(p->d_Yslab, kSlabs, stride, (size_t)nrhs * p->nbox * kNU, st));
-    if (uses_split(prec)) IE_TRY(launch_split_tc(p, (const float2 *)X, nrhs, is_fp16(prec), st));
-    IE_TRY(translate_timed(p, prec, (const float2 *)X, p->d_Yslab, nrhs, st, nullptr));
-    return launch_sum_slabs(p, p->d_Yslab, kSlabs, stride, (float2 *)Y, nrhs, st);
+    auto add = [&](int nslab, const int *form) {
+        return launch_sum_slabs(p, p->d_Yslab, nslab, slab_stride(p), (float2 *)Y, nrhs, st, form);
+    };
+    if (conv_far(p, prec)) return chosen_translate(p, prec, (const float2 *)X, nrhs, st, nullptr, add);
+    IE_TRY(block_translate(p, prec, (const float2 *)X, nrhs, st, nullptr));
+    return add(kSlabs, nullptr);
 }
 
 ie_status ie_disaggregate(ie_plan p, const void *Y, void *r, int nrhs, void *stream) {

@@ -9,7 +9,8 @@
 // and applies near blocks cut to |m|_inf <= 4 (no extra work), IE_FAR and ie_translate take
 // it off with the block-product kernels over the adjacent pairs (translate_simt.cu,
 // translate_tc.cu).  Nothing is added that cancels: all kept and removed terms have the
-// size of far interactions.
+// size of far interactions, as long as the sources are even enough (kFarEven); inputs that are
+// not take the block products.
 //
 // The convolution runs per scatterer and right-hand side over the scatterer's bounding
 // lattice (n_i = 4 E_i sites per axis, zero-padded to L_i >= 2 n_i - 1) in five passes:
@@ -621,8 +622,20 @@ constexpr double kPointNs = 0.03, kPairNs16 = 0.7, kBlockNs16 = 49, kPairNs32 = 
 // pairs 140 against 106 us in FP32).
 constexpr int64_t kFarPairs = 8192;
 constexpr size_t kConvWorkspace = (size_t)256 << 20;    // bytes of A and B beyond one column
+// The transforms round relative to the scatterer's whole field, a block product relative to what
+// reaches a box, and a far product leaves out what a box's own neighbourhood radiates.  So it is
+// a convolution only where, for every box and column, the far boxes hold at least 1 / kFarEven of
+// the sources' energy sum |x|^2: the worst box's rounding grows with the square root of that
+// ratio (6^3 boxes, one of them A above the rest, FP32: 4e-7 at A = 1, 7e-6 at 1e2, 7e-4 at 1e4;
+// blocks 5e-7 throughout).  Inputs that are not so even (a lone source, whose neighbourhood then
+// stays exactly zero, strong contrasts, NaN, infinities, or energies so large or small that a
+// transform's partial sums could leave FP32's range) take the block products, as decided on the
+// device for each call (launch_choose_form).  A plan in which even inputs already fail, because
+// some box has less than 1 / kFarEven of its scatterer far from it, keeps the blocks.
+constexpr double kFarEven = 4, kEnergyMin = 1e-60, kEnergyMax = 1e60;
 
-ConvUse conv_classes(const ie_problem *pr, int64_t npairs, int64_t nblocks, std::vector<ConvClass> &out) {
+ConvUse conv_classes(const ie_problem *pr, int64_t npairs, int64_t nblocks, const std::vector<int32_t> &near_start,
+                     std::vector<ConvClass> &out) {
     out.clear();
     unsigned mask = pr->prec_mask & kConvMask;
     if ((int64_t)pr->max_rhs * pr->n_boxes * kNU > (int64_t)INT32_MAX)   // the 16-bit forms' limit
@@ -676,7 +689,15 @@ ConvUse conv_classes(const ie_problem *pr, int64_t npairs, int64_t nblocks, std:
         const size_t per = (size_t)(c.a_col + c.b_col) * sizeof(float2);
         c.chunk = (int)std::min<int64_t>(std::min<int64_t>(cols, 16384), std::max<int64_t>(1, kConvWorkspace / per));
     }
-    return {mask, npairs >= kFarPairs ? mask : 0u};
+    bool even = true;       // with equal boxes every box has enough far sources
+    std::vector<int> boxes(G, 0);
+    for (int b = 0; b < pr->n_boxes; ++b) ++boxes[pr->box_group ? pr->box_group[b] : 0];
+    for (int b = 0; b < pr->n_boxes && even; ++b) {
+        const int n = boxes[pr->box_group ? pr->box_group[b] : 0];
+        const int near = near_start[b + 1] - near_start[b] + (pr->self_box_mode == 1 ? 1 : 0);
+        even = n <= kFarEven * (n - near);
+    }
+    return {mask, npairs >= kFarPairs && even ? mask : 0u};
 }
 
 size_t conv_bytes(const ie_problem *pr, const std::vector<ConvClass> &cl, const ConvUse &use, int64_t nadj,
@@ -701,6 +722,9 @@ size_t conv_bytes(const ie_problem *pr, const std::vector<ConvClass> &cl, const 
     if (pr->group_nrhs) add((size_t)pr->n_boxes * sizeof(int32_t));
     add(near_elems * sizeof(float2));                                   // short near blocks
     if (!use.far) return b;
+    add((size_t)pr->max_rhs * pr->n_boxes * sizeof(double));            // inputs' energies
+    add(((size_t)(pr->box_group ? pr->n_groups : 1) + 1) * sizeof(int32_t));
+    add(2 * sizeof(int));
     add(2 * (size_t)nadj * sizeof(int32_t));                            // adjacent pairs
     add((size_t)27 * kNU * kNU * sizeof(float2));                       // their masked blocks
     if (pr->prec_mask & (IE_PRECMASK(IE_PREC_BF16X3) | IE_PRECMASK(IE_PREC_FP16X3))) {
@@ -797,6 +821,92 @@ ie_status conv_create(ie_plan p, cudaStream_t st) {
     if (p->conv.empty()) return IE_OK;
     IE_TRY(dalloc_t(p, &p->d_convA, a));
     IE_TRY(dalloc_t(p, &p->d_convB, w));
+    return IE_OK;
+}
+
+namespace {
+
+// w[r][b] = sum_u |x_u|^2, a warp per box and column.  The squares are taken at a power of two near
+// the box's largest entry, so that neither overflows nor underflows.
+__global__ void __launch_bounds__(256) energy_kernel(const float2 *__restrict__ X, int64_t cols, double *__restrict__ w,
+                                                     int *__restrict__ form, const int *__restrict__ gate) {
+    const bool on = !gate || *gate != 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) form[0] = on, form[1] = 0;
+    const int64_t col = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (!on || col >= cols) return;
+    const int lane = threadIdx.x & 31;
+    float2 x[kNU / 32];
+    float m = 0.f;
+#pragma unroll
+    for (int t = 0; t < kNU / 32; ++t) {
+        x[t] = X[col * kNU + lane + 32 * t];
+        m = fmaxf(m, fmaxf(fabsf(x[t].x), fabsf(x[t].y)));
+    }
+    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    int e = 0;
+    if (m > 0.f && m <= 3.4028235e38f) frexpf(m, &e);   // NaN entries stay in the sum, infinite ones too
+    const float down = ldexpf(1.f, -(e / 2)), rest = ldexpf(1.f, e / 2 - e);
+    float s = 0.f;
+#pragma unroll
+    for (int t = 0; t < kNU / 32; ++t) {
+        const float a = x[t].x * down * rest, b = x[t].y * down * rest;
+        s = fmaf(a, a, fmaf(b, b, s));
+    }
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) w[col] = ldexp((double)s, 2 * e);
+}
+
+// A CTA takes kFormBoxes boxes of one scatterer and column, a warp four of them, lanes over the
+// stored near boxes (27 at most).  Every CTA sums the scatterer's energy itself, in one order.
+// Bound by its chain of reads.
+constexpr int kFormBoxes = 32;
+__global__ void __launch_bounds__(256) choose_form_kernel(const double *__restrict__ w, const int32_t *__restrict__ gbox,
+                                                          const int32_t *__restrict__ near_start,
+                                                          const int32_t *__restrict__ near_src,
+                                                          const int32_t *__restrict__ box_cols, int nbox,
+                                                          int *__restrict__ form, const int *__restrict__ gate) {
+    if (gate && *gate == 0) return;
+    __shared__ double red[8];
+    const int b0 = gbox[blockIdx.x], b1 = gbox[blockIdx.x + 1], first = b0 + (int)blockIdx.y * kFormBoxes;
+    const int r = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (first >= b1 || (box_cols && r >= box_cols[b0])) return;
+    const double *wr = w + (int64_t)r * nbox;
+    double near[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int t = min(first + 4 * warp + i, b1 - 1), q = near_start[t] + lane;
+        const int src = q < near_start[t + 1] ? near_src[q] : t;
+        near[i] = lane == 31 || src != t ? wr[src] : 0.0;       // lane 31 has no entry: the box itself
+    }
+    double s = 0;
+#pragma unroll 8
+    for (int b = b0 + threadIdx.x; b < b1; b += 256) s += wr[b];
+    for (int o = 16; o; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) near[i] += __shfl_xor_sync(0xffffffffu, near[i], o);
+    }
+    if (lane == 0) red[warp] = s;
+    __syncthreads();
+    s = ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
+    bool blocks = !(s == 0 || (s >= kEnergyMin && s <= kEnergyMax));        // NaN too
+#pragma unroll
+    for (int i = 0; i < 4; ++i) blocks |= !(s <= kFarEven * (s - near[i]));
+    if (blocks && lane == 0) form[0] = 0, form[1] = 1;       // one value from every warp
+}
+
+}  // namespace
+
+ie_status launch_choose_form(ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate) {
+    const int64_t cols = (int64_t)nrhs * p->nbox;
+    energy_kernel<<<(unsigned)((cols + 7) / 8), 256, 0, st>>>(X, cols, p->d_energy, p->d_form, gate);
+    IE_CK_LAUNCH();
+    int64_t most = 0;
+    for (int g = 0; g < p->ngroups; ++g) most = std::max(most, p->gbox[g + 1] - p->gbox[g]);
+    const dim3 grid(p->ngroups, (unsigned)((most + kFormBoxes - 1) / kFormBoxes), nrhs);
+    choose_form_kernel<<<grid, 256, 0, st>>>(
+        p->d_energy, p->d_gbox, p->d_near_start, p->d_near_src, p->d_box_cols, p->nbox, p->d_form, gate);
+    IE_CK_LAUNCH();
     return IE_OK;
 }
 

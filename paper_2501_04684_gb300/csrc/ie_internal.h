@@ -276,12 +276,15 @@ struct ie_plan_s {
     std::vector<ie::ConvClass> conv;
     ie::ConvUse conv_use;              // products that take it
     float2 *d_convA = nullptr, *d_convB = nullptr;
-    cudaStream_t side = nullptr;       // the near part of a full product runs beside the convolution
+    cudaStream_t side = nullptr;       // runs beside the convolution (near part, choice of a far product's form)
     cudaEvent_t fork = nullptr, join = nullptr;
     int32_t *d_box_cols = nullptr;     // [nbox] right-hand sides of each box's scatterer (null: all)
     float2 *d_Nshort = nullptr;        // near blocks of the site pairs within kNearReach (as d_Nblk)
     // adjacent pairs (26 groups) whose site pairs beyond kNearReach the convolution holds,
     // with the negated blocks of just those site pairs
+    int32_t *d_gbox = nullptr;         // [ngroups + 1] box range of each scatterer
+    double *d_energy = nullptr;        // [max_rhs][nbox] sum |x_u|^2 of a far product's inputs
+    int *d_form = nullptr;             // the far product's form: convolution, blocks (one of them 1)
     int64_t n_adj = 0;
     std::vector<int64_t> h_adj_start;  // 28 (groups e = (ex+1)*9 + (ey+1)*3 + (ez+1))
     std::vector<int32_t> h_adj_src;    // kept only with gnrhs
@@ -336,11 +339,16 @@ ie_status launch_near_blocks(ie_plan p, cudaStream_t st);
 
 // ---- far product as a lattice convolution (conv.cu)
 // the classes of a problem's scatterers (nblocks: stored blocks its pairs use) and what they serve
-ConvUse conv_classes(const ie_problem *pr, int64_t npairs, int64_t nblocks, std::vector<ConvClass> &out);
+// (near_start: the near lists' offsets)
+ConvUse conv_classes(const ie_problem *pr, int64_t npairs, int64_t nblocks, const std::vector<int32_t> &near_start,
+                     std::vector<ConvClass> &out);
 size_t conv_bytes(const ie_problem *pr, const std::vector<ConvClass> &cl, const ConvUse &use, int64_t nadj,
                   int64_t near_elems);
 int64_t conv_traffic(const ie_plan_s *p, int nrhs);
 ie_status conv_create(ie_plan p, cudaStream_t st);
+// Sets p->d_form for the inputs X of a far product (see kFarEven): the entry of the form that
+// serves them to 1, the other to 0; both to 0 when `gate` reads 0.
+ie_status launch_choose_form(ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate);
 // Y = K' * X at every box (zero in columns a scatterer does not have)
 ie_status launch_conv(ie_plan p, const float2 *X, float2 *Y, int nrhs, cudaStream_t st, const int *gate);
 inline bool conv_full(const ie_plan_s *p, int prec) { return (p->conv_use.full & IE_PRECMASK(prec)) != 0; }
@@ -352,24 +360,29 @@ ie_status adj_list(ie_plan p, bool tc, int nrhs, WorkList **out);
 ie_status launch_aggregate(const ie_plan p, const float2 *c, float2 *X, int nrhs, cudaStream_t st,
                            const int *gate = nullptr);
 // symmetry = 1: the 48 signed-permuted FP32 copies of X into p->d_Xsym
-ie_status launch_permute_sym(const ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate = nullptr);
+// most_ctas here and below: at most so many CTAs (per column) that loop, for launches that are
+// mostly gated off
+ie_status launch_permute_sym(const ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate = nullptr,
+                             int most_ctas = INT32_MAX);
 // plain: without the symmetric store's permuted copies
 ie_status launch_split_tc(const ie_plan p, const float2 *X, int nrhs, bool fp16, cudaStream_t st,
-                          const int *gate = nullptr, bool plain = false);
+                          const int *gate = nullptr, bool plain = false, int most_ctas = INT32_MAX);
+// form (p->d_form, may be null): nslab slabs in the convolution's form, kSlabs in the blocks'
 ie_status launch_disaggregate(const ie_plan p, const float2 *Yslab, int nslab, size_t slab_stride, float2 *r,
-                              int nrhs, bool accumulate, cudaStream_t st, const int *gate = nullptr);
+                              int nrhs, bool accumulate, cudaStream_t st, const int *gate = nullptr,
+                              const int *form = nullptr);
 ie_status launch_sum_slabs(const ie_plan p, const float2 *Yslab, int nslab, size_t slab_stride, float2 *Y, int nrhs,
-                           cudaStream_t st);
+                           cudaStream_t st, const int *form = nullptr);
 ie_status launch_zero(void *ptr, size_t bytes, cudaStream_t st, const int *gate = nullptr);
 // nslab regions of `count` complex values, `stride` complex values apart, in one launch
 ie_status launch_zero_slabs(float2 *base, int nslab, size_t stride, size_t count, cudaStream_t st,
-                            const int *gate = nullptr);
+                            const int *gate = nullptr, int most_ctas = INT32_MAX);
 // shorter: only the site pairs within kNearReach (the others are in the convolution);
 // most_ctas: leave the rest of the GPU to kernels that run beside it
 ie_status launch_near(const ie_plan p, const float2 *c, float2 *y, int nrhs, cudaStream_t st,
                       const int *gate = nullptr, bool shorter = false, int most_ctas = INT32_MAX);
 ie_status launch_translate_simt(ie_plan p, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
-                                const int *gate = nullptr, bool adjacent = false);
+                                const int *gate = nullptr, bool adjacent = false, int most_ctas = INT32_MAX);
 ie_status launch_translate_cvfcnn(ie_plan p, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
                                   const int *gate = nullptr);
 // fits the surrogates of the ncanon canonical displacements (device, ncanon x 3); with
@@ -412,9 +425,6 @@ void store_retain(ie_store s);
 void store_release(ie_store s);
 int cvfcnn_tc_tile_columns();
 void destroy_cached_solvers(ie_plan p);
-// launch the translation kernel of `prec` (with the profiling brackets when enabled)
-ie_status translate_timed(ie_plan p, int prec, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
-                          const int *gate);
 int simt_tile_columns();
 int tc_tile_columns();
 // runs one bounded device wait on an mbarrier nothing signals (IE_ERR_TIMEOUT expected)

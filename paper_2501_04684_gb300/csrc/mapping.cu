@@ -5,6 +5,8 @@
 // Layouts: c, r: [rhs][n] complex64 (box b's coefficients at off[b] .. off[b+1]);
 // P: [n][192] complex64 (row off[b]+i is basis function i of box b);
 // X, Y: [rhs][nbox][192] complex64.  All HBM-bound: one CTA per box and up to four columns.
+#include <algorithm>
+
 #include "ie_internal.h"
 
 namespace ie {
@@ -81,12 +83,11 @@ constexpr int kSplitCopies = 8;
 static_assert(kNU / 8 * kSplitCopies == kNU, "one thread per eight unknowns of a copy");
 static_assert(kSym % kSplitCopies == 0, "whole groups of copies");
 template <bool FP16>
-__global__ void __launch_bounds__(kNU)
-split_kernel(const float2 *__restrict__ X, int nbox, int nrhs, uint16_t *__restrict__ Xtc, int32_t *__restrict__ Xexp,
-             float *__restrict__ Xinf, const uint16_t *__restrict__ symmap, const int *__restrict__ gate) {
-    if (gate && *gate == 0) return;
+__device__ __forceinline__ void split_column(int b, const float2 *__restrict__ X, int nbox, int nrhs,
+                                             uint16_t *__restrict__ Xtc, int32_t *__restrict__ Xexp,
+                                             float *__restrict__ Xinf, const uint16_t *__restrict__ symmap) {
     __shared__ uint2 halves[kNU];           // (hi re, hi im), (lo re, lo im)
-    const int b = blockIdx.x, r = blockIdx.y, u = threadIdx.x;
+    const int r = blockIdx.y, u = threadIdx.x;
     const int64_t col = (int64_t)r * nbox + b;
     const float2 x = X[col * kNU + u];
     const bool write_exp = blockIdx.z == 0;
@@ -173,6 +174,17 @@ split_kernel(const float2 *__restrict__ X, int nbox, int nrhs, uint16_t *__restr
     }
 }
 
+template <bool FP16>
+__global__ void __launch_bounds__(kNU)
+split_kernel(const float2 *__restrict__ X, int nbox, int nrhs, uint16_t *__restrict__ Xtc, int32_t *__restrict__ Xexp,
+             float *__restrict__ Xinf, const uint16_t *__restrict__ symmap, const int *__restrict__ gate) {
+    if (gate && *gate == 0) return;
+    for (int b = blockIdx.x; b < nbox; b += gridDim.x) {
+        if (b != (int)blockIdx.x) __syncthreads();      // the column before has been read
+        split_column<FP16>(b, X, nbox, nrhs, Xtc, Xexp, Xinf, symmap);
+    }
+}
+
 // Sum of an entry's nslab <= kSlabs partial sums (FP64), their reads in flight together.
 __device__ __forceinline__ float2 slab_sum(const float2 *__restrict__ Y, int nslab, size_t slab_stride) {
     float2 w[kSlabs];
@@ -187,6 +199,14 @@ __device__ __forceinline__ float2 slab_sum(const float2 *__restrict__ Y, int nsl
     return make_float2((float)sr, (float)si);
 }
 
+// A far product's slabs in the form it took (p->d_form): nslab as given, or the blocks' kSlabs.
+// False where it took neither (gated off).
+__device__ __forceinline__ bool form_slabs(const int *__restrict__ form, int &nslab) {
+    const int conv = form[0], blocks = form[1];
+    if (blocks) nslab = kSlabs;
+    return conv || blocks;
+}
+
 // r[i] (+)= sum_u P[i][u] y[u], y = sum over slabs (FP64), for NR right-hand sides (P is read
 // once for them).  A warp takes four basis rows at a time, lanes over u, all 24 reads of P in
 // flight; FP32 products and a tree that halves the number of sums a lane carries at each step
@@ -199,9 +219,10 @@ __global__ void __launch_bounds__(kDisThreads) disaggregate_kernel(const float2 
                                                            const int64_t *__restrict__ off, int64_t n, int nbox,
                                                            const float2 *__restrict__ Yslab, int nslab,
                                                            size_t slab_stride, float2 *__restrict__ out, int accumulate,
-                                                           int identity, int nrhs, const int *__restrict__ gate) {
-    chain_next();
+                                                           int identity, int nrhs, const int *__restrict__ gate,
+                                                           const int *__restrict__ form) {
     if (gate && *gate == 0) return;
+    if (form && !form_slabs(form, nslab)) return;
     constexpr int kRows = 4, M = 2 * kRows * NR;
     __shared__ float2 ys[NR][kNU];
     const int b = blockIdx.x, r0 = blockIdx.y * NR;
@@ -307,7 +328,8 @@ __global__ void zero_slabs_kernel(float4 *__restrict__ p, int64_t n4, int64_t st
 }
 
 __global__ void sum_slabs_kernel(const float2 *__restrict__ Yslab, int nslab, size_t slab_stride, int64_t count,
-                                 float2 *__restrict__ Y) {
+                                 float2 *__restrict__ Y, const int *__restrict__ form) {
+    if (form && !form_slabs(form, nslab)) return;
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     Y[i] = slab_sum(Yslab + i, nslab, slab_stride);
@@ -386,9 +408,9 @@ ie_status launch_aggregate(const ie_plan p, const float2 *c, float2 *X, int nrhs
 }
 
 ie_status launch_split_tc(const ie_plan p, const float2 *X, int nrhs, bool fp16, cudaStream_t st, const int *gate,
-                          bool plain) {
+                          bool plain, int most_ctas) {
     const bool sym = p->sym && !plain;
-    const dim3 grid(p->nbox, nrhs, sym ? kSym / kSplitCopies : 1);
+    const dim3 grid(std::min(p->nbox, most_ctas), nrhs, sym ? kSym / kSplitCopies : 1);
     const uint16_t *map = sym ? p->d_symmap : nullptr;
     if (fp16)
         split_kernel<true><<<grid, kNU, 0, st>>>(X, p->nbox, nrhs, p->d_Xtc, p->d_Xexp, p->d_Xinf, map, gate);
@@ -403,26 +425,28 @@ ie_status launch_split_tc(const ie_plan p, const float2 *X, int nrhs, bool fp16,
 __global__ void permute_sym_kernel(const float2 *__restrict__ X, int nbox, int nrhs, const uint16_t *__restrict__ symmap,
                                    float2 *__restrict__ Xsym, const int *__restrict__ gate) {
     if (gate && *gate == 0) return;
-    const int b = blockIdx.x, r = blockIdx.y, sg = blockIdx.z, u = threadIdx.x;
-    const int64_t col = (int64_t)r * nbox + b;
+    const int r = blockIdx.y, sg = blockIdx.z, u = threadIdx.x;
     const uint16_t e = symmap[sg * kNU + u];
-    float2 x = X[col * kNU + (e & 0xFF)];
-    if (e & 0x100) x = make_float2(-x.x, -x.y);
-    Xsym[((int64_t)sg * nrhs * nbox + col) * kNU + u] = x;
+    for (int b = blockIdx.x; b < nbox; b += gridDim.x) {
+        const int64_t col = (int64_t)r * nbox + b;
+        float2 x = X[col * kNU + (e & 0xFF)];
+        if (e & 0x100) x = make_float2(-x.x, -x.y);
+        Xsym[((int64_t)sg * nrhs * nbox + col) * kNU + u] = x;
+    }
 }
 
-ie_status launch_permute_sym(const ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate) {
-    permute_sym_kernel<<<dim3(p->nbox, nrhs, kSym), kNU, 0, st>>>(X, p->nbox, nrhs, p->d_symmap, p->d_Xsym, gate);
+ie_status launch_permute_sym(const ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate, int most_ctas) {
+    permute_sym_kernel<<<dim3(std::min(p->nbox, most_ctas), nrhs, kSym), kNU, 0, st>>>(X, p->nbox, nrhs, p->d_symmap, p->d_Xsym, gate);
     IE_CK_LAUNCH();
     return IE_OK;
 }
 
 ie_status launch_disaggregate(const ie_plan p, const float2 *Yslab, int nslab, size_t stride, float2 *r, int nrhs,
-                              bool accumulate, cudaStream_t st, const int *gate) {
+                              bool accumulate, cudaStream_t st, const int *gate, const int *form) {
 #define IE_DIS(NR)                                                                                                 \
     disaggregate_kernel<NR><<<dim3(p->nbox, (nrhs + NR - 1) / NR), kDisThreads, 0, st>>>(                          \
         p->d_P, p->d_nb, p->d_off, p->n, p->nbox, Yslab, nslab, stride, r, accumulate ? 1 : 0, p->identity ? 1 : 0, \
-        nrhs, gate)
+        nrhs, gate, form)
     if (nrhs == 1)
         IE_DIS(1);
     else if (nrhs == 2)
@@ -448,7 +472,8 @@ ie_status launch_zero(void *ptr, size_t bytes, cudaStream_t st, const int *gate)
     return IE_OK;
 }
 
-ie_status launch_zero_slabs(float2 *base, int nslab, size_t stride, size_t count, cudaStream_t st, const int *gate) {
+ie_status launch_zero_slabs(float2 *base, int nslab, size_t stride, size_t count, cudaStream_t st, const int *gate,
+                            int most_ctas) {
     if (count == 0 || nslab == 0) return IE_OK;
     if ((count * sizeof(float2)) % 16 || (stride * sizeof(float2)) % 16) {
         set_error("launch_zero_slabs: sizes not multiples of 16 bytes");
@@ -456,7 +481,7 @@ ie_status launch_zero_slabs(float2 *base, int nslab, size_t stride, size_t count
     }
     const int64_t n4 = (int64_t)(count * sizeof(float2) / 16);
     int64_t gx = (n4 + 255) / 256;
-    if (gx > 1024) gx = 1024;
+    gx = std::min<int64_t>(gx, std::min(1024, most_ctas));
     zero_slabs_kernel<<<dim3((unsigned)gx, (unsigned)nslab), 256, 0, st>>>(reinterpret_cast<float4 *>(base), n4,
                                                                           (int64_t)(stride * sizeof(float2) / 16),
                                                                           gate);
@@ -465,9 +490,9 @@ ie_status launch_zero_slabs(float2 *base, int nslab, size_t stride, size_t count
 }
 
 ie_status launch_sum_slabs(const ie_plan p, const float2 *Yslab, int nslab, size_t stride, float2 *Y, int nrhs,
-                           cudaStream_t st) {
+                           cudaStream_t st, const int *form) {
     int64_t count = (int64_t)nrhs * p->nbox * kNU;
-    sum_slabs_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(Yslab, nslab, stride, count, Y);
+    sum_slabs_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(Yslab, nslab, stride, count, Y, form);
     IE_CK_LAUNCH();
     return IE_OK;
 }

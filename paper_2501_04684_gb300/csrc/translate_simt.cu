@@ -13,6 +13,7 @@
 // of different displacements meet in one of kSlabs FP32 partial fields (slab =
 // d mod kSlabs, red.global.add.v4.f32), and the slabs are added in FP64 by the
 // inverse-mapping kernel, so no FP32 sum runs over more than ~N_far/kSlabs terms.
+#include <algorithm>
 #include <mutex>
 
 #include "ie_internal.h"
@@ -177,9 +178,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 translate_simt_kernel(const WorkItem *__restrict__ items, const float2 *__restrict__ C,
                       const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
                       const float2 *__restrict__ X, float2 *__restrict__ Yslab, size_t slab_stride,
-                      int nbox, int nrhs, const SymArgs sy, const int *__restrict__ gate) {
+                      int nbox, int nrhs, const SymArgs sy, unsigned n_items, const int *__restrict__ gate) {
     if (gate && *gate == 0) return;
-    simt_tile(items[blockIdx.x], C, src, dst, X, Yslab, slab_stride, nbox, nrhs, sy);
+    // (a tile's last reads of shared memory are behind its last barrier)
+    for (unsigned i = blockIdx.x; i < n_items; i += gridDim.x)
+        simt_tile(items[i], C, src, dst, X, Yslab, slab_stride, nbox, nrhs, sy);
 }
 
 }  // namespace
@@ -193,13 +196,14 @@ ie_status prepare_translate_simt() {
 }
 
 ie_status launch_translate_simt(ie_plan p, const float2 *X, float2 *Yslab, int nrhs, cudaStream_t st,
-                                const int *gate, bool adjacent) {
+                                const int *gate, bool adjacent, int most_ctas) {
     WorkList *wl = nullptr;
     if (adjacent) {     // one block per displacement, at most 26 terms per target: one slab
         IE_TRY(adj_list(p, false, nrhs, &wl));
         if (wl->n == 0) return IE_OK;
         translate_simt_kernel<<<(unsigned)wl->n, kThreads, sizeof(SmemSimt), st>>>(
-            wl->d_items, p->d_Cadj, p->d_adj_src, p->d_adj_dst, X, Yslab, 0, p->nbox, nrhs, SymArgs(), gate);
+            wl->d_items, p->d_Cadj, p->d_adj_src, p->d_adj_dst, X, Yslab, 0, p->nbox, nrhs, SymArgs(),
+            (unsigned)wl->n, gate);
         IE_CK_LAUNCH();
         return IE_OK;
     }
@@ -208,7 +212,7 @@ ie_status launch_translate_simt(ie_plan p, const float2 *X, float2 *Yslab, int n
     if (!p->d_Csimt) return set_error("the plan holds no FP32 coupling store"), IE_ERR_UNSUPPORTED;
     SymArgs sy;
     if (p->sym) {
-        IE_TRY(launch_permute_sym(p, X, nrhs, st, gate));
+        IE_TRY(launch_permute_sym(p, X, nrhs, st, gate, most_ctas));
         X = p->d_Xsym;
         sy.gcanon = p->d_gcanon;
         sy.gsigma = p->d_gsigma;
@@ -216,8 +220,8 @@ ie_status launch_translate_simt(ie_plan p, const float2 *X, float2 *Yslab, int n
         sy.map = p->d_symmap;
         sy.stride = (size_t)nrhs * p->nbox * kNU;
     }
-    translate_simt_kernel<<<(unsigned)wl->n, kThreads, sizeof(SmemSimt), st>>>(
-        wl->d_items, p->d_Csimt, p->d_src, p->d_dst, X, Yslab, slab_stride(p), p->nbox, nrhs, sy, gate);
+    translate_simt_kernel<<<(unsigned)std::min<int64_t>(wl->n, most_ctas), kThreads, sizeof(SmemSimt), st>>>(
+        wl->d_items, p->d_Csimt, p->d_src, p->d_dst, X, Yslab, slab_stride(p), p->nbox, nrhs, sy, (unsigned)wl->n, gate);
     IE_CK_LAUNCH();
     return IE_OK;
 }
