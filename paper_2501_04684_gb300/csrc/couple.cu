@@ -233,7 +233,8 @@ near_blocks_kernel(const float2 *__restrict__ Cnear,     // [27 or 54][k][m], in
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     S.W[2 * tm + 64 * (i >> 1) + (i & 1)][4 * tn + j] =
-                        make_float2(hi[i][j].x + lo[i][j].x, hi[i][j].y + lo[i][j].y);
+                        make_float2(two_float_total(hi[i][j].x, lo[i][j].x),
+                                    two_float_total(hi[i][j].y, lo[i][j].y));
             __syncthreads();
             // N[i][j0 + jj] = sum_m Pa[i][m] W[m][jj]: lane = column, a warp takes four rows at a time
             const int jj = tid & 31, warp = tid >> 5;
@@ -264,7 +265,8 @@ near_blocks_kernel(const float2 *__restrict__ Cnear,     // [27 or 54][k][m], in
 #pragma unroll
                 for (int r = 0; r < 4; ++r)
                     if (i0 + r < na && jj < nj) {
-                        const float2 v = make_float2(h[r].x + l[r].x, h[r].y + l[r].y);
+                        const float2 v =
+                            make_float2(two_float_total(h[r].x, l[r].x), two_float_total(h[r].y, l[r].y));
                         N[(int64_t)(j0 + jj) * na + i0 + r] = v;
                         if (Nshort && e == 13) Nshort[boff[pi] + (int64_t)(j0 + jj) * na + i0 + r] = v;
                     }

@@ -86,13 +86,20 @@ __device__ inline void dyad_fp64(double k, double eta, double Rx, double Ry, dou
         }
 }
 
-// (hi, lo) += x without losing the rounding of the sum: FP32 chunk sums kept to twice FP32's
-// digits at FP32 rate (an FP64 addition takes the issue time of 64 FP32 ones on this GPU).
+// (hi, lo) += x / 16 without losing the rounding of the sum: FP32 partial sums kept to twice
+// FP32's digits at FP32 rate (an FP64 addition takes the issue time of 64 FP32 ones on this GPU).
+// At most 16 terms: the total is held at a sixteenth, so that finite terms cannot overflow it, and
+// lo counts only while hi is finite: two_float_total gives what an FP64 total would (rounded to
+// FP32: infinite out of range).
+constexpr int kTotalTerms = 16;
 __device__ __forceinline__ void two_float_add(float &hi, float &lo, float x) {
-    const float s = hi + x, b = s - hi;
-    lo += (hi - (s - b)) + (x - b);
+    constexpr float c = 1.f / kTotalTerms;
+    const float s = fmaf(x, c, hi), b = s - hi;
+    lo += (hi - (s - b)) + fmaf(x, c, -b);
     hi = s;
 }
+__device__ __forceinline__ float low_of(float hi, float lo) { return fabsf(hi) <= 3.402823466e38f ? lo : 0.f; }
+__device__ __forceinline__ float two_float_total(float hi, float lo) { return kTotalTerms * (hi + low_of(hi, lo)); }
 
 void set_error(const char *fmt, ...);
 const char *last_error();

@@ -58,7 +58,9 @@ __global__ void __launch_bounds__(kNU) aggregate_kernel(const float2 *__restrict
     }
 #pragma unroll
     for (int r = 0; r < NR; ++r)
-        if (r0 + r < nrhs) X[((int64_t)(r0 + r) * nbox + b) * kNU + u] = make_float2(hi[r].x + lo[r].x, hi[r].y + lo[r].y);
+        if (r0 + r < nrhs)
+            X[((int64_t)(r0 + r) * nbox + b) * kNU + u] =
+                make_float2(two_float_total(hi[r].x, lo[r].x), two_float_total(hi[r].y, lo[r].y));
 }
 
 __global__ void copy_kernel(const float4 *__restrict__ a, float4 *__restrict__ b, int64_t n4,
