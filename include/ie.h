@@ -406,7 +406,8 @@ ie_status ie_solve(ie_plan plan, const void *v, void *c, int nrhs, const ie_solv
  * right-hand sides on `plan` (refine must be 0). */
 ie_status ie_solver_create(ie_plan plan, int nrhs, const ie_solve_opts *opts, ie_solver *out);
 
-/* Device bytes ie_solver_create would allocate. */
+/* Device bytes ie_solver_create would allocate; with opts->refine those that a refined
+ * ie_solve keeps with the plan: its inner solver and the refinement's vectors. */
 ie_status ie_solver_footprint(ie_plan plan, int nrhs, const ie_solve_opts *opts, size_t *bytes);
 
 /* Enqueue the start of a solve of Z c = v (x0 = 0); v and c must stay valid until

@@ -721,7 +721,7 @@ ie_status salloc_t(ie_solver s, T **p, size_t count) {
     return salloc(s, reinterpret_cast<void **>(p), count * sizeof(T));
 }
 
-size_t solver_bytes(int64_t n, int R, int G, int m, int C, int nblk) {
+size_t solver_bytes(int64_t n, int R, int G, int m, int C, int nblk, bool refine) {
     const int64_t S = (int64_t)R * G;
     size_t b = 0;
     b += (size_t)(m + 1) * R * n * sizeof(float2);           // V
@@ -732,6 +732,10 @@ size_t solver_bytes(int64_t n, int R, int G, int m, int C, int nblk) {
     b += (size_t)S * (m + 1) * nblk * sizeof(double2);       // partial
     b += (size_t)S * 2 * sizeof(double) + (6 + 5 * S + 2) * sizeof(int);   // bnorm, status, counters
     b += (size_t)C * (2 * sizeof(int32_t) + sizeof(int64_t)) + (size_t)(G + 1) * sizeof(int64_t) + G * sizeof(int32_t);
+    if (refine) {      // refinement_buffers
+        b += (size_t)R * n * (sizeof(double2) + 3 * sizeof(float2));
+        b += (size_t)S * nblk * sizeof(double2);
+    }
     return b;
 }
 
@@ -961,7 +965,7 @@ ie_status ie_solver_footprint(ie_plan p, int nrhs, const ie_solve_opts *opts, si
     fill_defaults(&o);
     if (opts) o = *opts;
     Chunks c = make_chunks(p);
-    *bytes = solver_bytes(p->n, nrhs, p->ngroups, o.restart, (int)c.group.size(), c.nblk);
+    *bytes = solver_bytes(p->n, nrhs, p->ngroups, o.restart, (int)c.group.size(), c.nblk, o.refine != 0);
     return IE_OK;
 }
 
