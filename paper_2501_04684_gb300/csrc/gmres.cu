@@ -923,6 +923,7 @@ ie_status mirror_status(ie_solver s, cudaStream_t st) {
 // then allocates nothing, and the captured cycle's pointers stay the same from call to call.
 ie_status refinement_buffers(ie_solver s) {
     if (s->h_part) return IE_OK;
+    std::lock_guard<std::recursive_mutex> lock(device_mutex());
     const size_t total = (size_t)s->R * s->n, np = (size_t)s->S * s->nblk;
     if (!s->x64) IE_TRY(salloc_t(s, &s->x64, total));
     if (!s->rv) IE_TRY(salloc_t(s, &s->rv, total));
