@@ -654,7 +654,8 @@ namespace ie {
 namespace {
 // One CTA per stored network: the inference layout (W1^T [192][64], b1, W2^T [64][192], b2)
 // to the caller's (W1 [H][192], b1 [H], W2 [192][H], b2 [192]).  The host loop this replaces
-// took 4 ms for 146 networks.
+// took 4 ms for 146 networks.  In chunks: the networks of a plan may be most of the device's memory.
+constexpr size_t kUnpackBytes = (size_t)8 << 20;
 __global__ void cvfcnn_unpack_kernel(const float2 *__restrict__ W, int H, float2 *__restrict__ W1,
                                      float2 *__restrict__ b1, float2 *__restrict__ W2, float2 *__restrict__ b2) {
     const float2 *o = W + (size_t)blockIdx.x * kCvBlockElems;
@@ -675,24 +676,32 @@ extern "C" ie_status ie_cvfcnn_get_weights(ie_plan p, float *W1, float *b1, floa
     if (!p->d_cvW) return set_error("the plan holds no CVFCNN surrogates"), IE_ERR_UNSUPPORTED;
     const size_t H = p->cv_hidden, nblk = p->n_blocks;
     if (nblk == 0) return IE_OK;
-    const size_t n1 = nblk * H * kNU, c1 = nblk * H, c2 = nblk * kNU;
+    const size_t n1 = H * kNU, net = 2 * n1 + H + kNU;      // complex values of one network
     cudaStream_t st = (cudaStream_t)stream;
-    float2 *d = nullptr;        // the caller's four arrays one after the other
-    if (cudaMallocAsync(&d, (2 * n1 + c1 + c2) * sizeof(float2), st) != cudaSuccess) {
+    // 8 MB of scratch or fewer (one network takes at most 200 KB)
+    size_t chunk = std::min<size_t>(nblk, std::max<size_t>(1, kUnpackBytes / (net * sizeof(float2))));
+    float2 *d = nullptr;        // a chunk's four arrays one after the other
+    while (cudaMallocAsync(&d, chunk * net * sizeof(float2), st) != cudaSuccess) {
         cudaGetLastError();
-        return set_error("network read-back scratch (%zu networks)", nblk), IE_ERR_OOM;
+        if (chunk == 1) return set_error("network read-back scratch"), IE_ERR_OOM;
+        chunk = (chunk + 1) / 2;
     }
-    float2 *dW1 = d, *dW2 = d + n1, *db1 = dW2 + n1, *db2 = db1 + c1;
-    cvfcnn_unpack_kernel<<<(unsigned)nblk, 256, 0, st>>>(p->d_cvW, (int)H, dW1, db1, dW2, db2);
-    count_launches(1);
-    cudaError_t e = cudaGetLastError();
-    auto copy = [&](float *to, const float2 *from, size_t n) {
-        if (e == cudaSuccess) e = cudaMemcpyAsync(to, from, n * sizeof(float2), cudaMemcpyDeviceToHost, st);
-    };
-    copy(W1, dW1, n1);
-    copy(b1, db1, c1);
-    copy(W2, dW2, n1);
-    copy(b2, db2, c2);
+    cudaError_t e = cudaSuccess;
+    for (size_t c0 = 0; c0 < nblk && e == cudaSuccess; c0 += chunk) {
+        const size_t m = std::min(chunk, nblk - c0);
+        float2 *dW1 = d, *dW2 = d + m * n1, *db1 = dW2 + m * n1, *db2 = db1 + m * H;
+        cvfcnn_unpack_kernel<<<(unsigned)m, 256, 0, st>>>(p->d_cvW + c0 * kCvBlockElems, (int)H, dW1, db1, dW2, db2);
+        count_launches(1);
+        e = cudaGetLastError();
+        auto copy = [&](float *to, const float2 *from, size_t per) {
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(to + 2 * c0 * per, from, m * per * sizeof(float2), cudaMemcpyDeviceToHost, st);
+        };
+        copy(W1, dW1, n1);
+        copy(b1, db1, H);
+        copy(W2, dW2, n1);
+        copy(b2, db2, kNU);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFreeAsync(d, st);
     if (e != cudaSuccess) return set_error("network read-back: %s", cudaGetErrorString(e)), IE_ERR_CUDA;
