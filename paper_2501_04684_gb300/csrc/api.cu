@@ -756,8 +756,10 @@ static ie_status check_store(const ie_problem *pr, ie_store store) {
     return IE_OK;
 }
 
-static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream, ie_plan *out) {
-    ie::NvtxRange nvtx_range("ie_plan_create");
+// conv: whether the far products may be convolutions; on return, whether some are.
+static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream, bool &conv, ie_plan *out) {
+    const bool allowed = conv;
+    conv = false;
     auto t0 = std::chrono::steady_clock::now();
     if (!out) return set_error("null out"), IE_ERR_INVALID;
     *out = nullptr;
@@ -1036,8 +1038,9 @@ static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream,
     }
 
     // far product as a convolution: its blocks of the adjacent pairs, K^, workspace
-    p->conv_use = conv_classes(pr, p->n_far_pairs, p->sym ? ncanon_used : p->n_far_disp, nstart, p->conv);
+    if (allowed) p->conv_use = conv_classes(pr, p->n_far_pairs, p->sym ? ncanon_used : p->n_far_disp, nstart, p->conv);
     if (!p->conv.empty()) {
+        conv = true;
         PT(conv_create(p, st));
         PC(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking));
         PC(cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming));
@@ -1108,6 +1111,17 @@ static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream,
     return IE_OK;
 #undef PT
 #undef PC
+}
+
+// A plan that does not fit with the convolution's arrays (its workspace, K^ and the near blocks'
+// second set) is made without them.
+static ie_status plan_create(const ie_problem *pr, ie_store store, void *stream, ie_plan *out) {
+    ie::NvtxRange nvtx_range("ie_plan_create");
+    bool conv = true;
+    const ie_status s = plan_create(pr, store, stream, conv, out);
+    if (s != IE_ERR_OOM || !conv) return s;
+    conv = false;
+    return plan_create(pr, store, stream, conv, out);
 }
 
 extern "C" {

@@ -756,9 +756,9 @@ ie_status build_khat(ie_plan p, ConvClass &c, cudaStream_t st) {
     IE_CK(cudaMemcpy(c.d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice));
     ie_status rc = IE_OK;
     auto body = [&]() -> ie_status {
-        IE_CK(cudaMallocAsync(&t0, s0 * sizeof(double2), st));
-        IE_CK(cudaMallocAsync(&t1, s1 * sizeof(double2), st));
-        IE_CK(cudaMallocAsync(&cs, h.size() * sizeof(double), st));
+        IE_TRY(scratch_alloc(&t0, s0, st));
+        IE_TRY(scratch_alloc(&t1, s1, st));
+        IE_TRY(scratch_alloc(&cs, h.size(), st));
         IE_CK(cudaMemcpyAsync(cs, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice, st));
         const double *ct[3] = {cs, cs + c.L[0], cs + c.L[0] + c.L[1]};
         int comp = 0;

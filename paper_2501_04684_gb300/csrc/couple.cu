@@ -334,9 +334,14 @@ ie_status launch_near_blocks(ie_plan p, cudaStream_t st) {
     int32_t *d_ds = nullptr;
     float2 *d_C = nullptr;
     int32_t *d_pa = nullptr;
-    IE_CK(cudaMallocAsync(&d_ds, ds.size() * sizeof(int32_t), st));
-    IE_CK(cudaMallocAsync(&d_C, (size_t)54 * kNU * kNU * sizeof(float2), st));
-    IE_CK(cudaMallocAsync(&d_pa, (size_t)p->n_near_pairs * sizeof(int32_t), st));
+    ie_status room = scratch_alloc(&d_ds, ds.size(), st);
+    if (room == IE_OK) room = scratch_alloc(&d_C, (size_t)54 * kNU * kNU, st);
+    if (room == IE_OK) room = scratch_alloc(&d_pa, (size_t)p->n_near_pairs, st);
+    if (room != IE_OK) {
+        for (void *q : {(void *)d_ds, (void *)d_C})
+            if (q) cudaFreeAsync(q, st);
+        return room;
+    }
     IE_CK(cudaMemcpyAsync(d_ds, ds.data(), ds.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     IE_TRY(launch_coupling_simt(p, d_ds, 27, d_C, false, st));
     if (p->d_Nshort)

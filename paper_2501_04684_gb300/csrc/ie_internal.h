@@ -335,6 +335,17 @@ ie_status dalloc_t(ie_plan p, T **ptr, size_t count) {
     return dalloc(p, reinterpret_cast<void **>(ptr), count * sizeof(T));
 }
 
+// Stream-ordered scratch of a set-up step: IE_ERR_OOM (and a null pointer) where there is none.
+template <class T>
+ie_status scratch_alloc(T **ptr, size_t count, cudaStream_t st) {
+    const cudaError_t e = cudaMallocAsync(ptr, count * sizeof(T), st);
+    if (e == cudaSuccess) return IE_OK;
+    cudaGetLastError();
+    *ptr = nullptr;
+    set_error("scratch of %zu bytes: %s", count * sizeof(T), cudaGetErrorString(e));
+    return e == cudaErrorMemoryAllocation ? IE_ERR_OOM : IE_ERR_CUDA;
+}
+
 // kernels (launchers), each stream-ordered.  `gate` (device int, may be null): when
 // it reads 0 the kernels return at once (used by GMRES after convergence).
 ie_status prepare_kernels();

@@ -1,4 +1,4 @@
-"""Device memory of solvers and network read-back."""
+"""Device memory of solvers, network read-back and plans."""
 import ctypes
 import glob
 import os
@@ -9,6 +9,7 @@ import torch
 
 import paper_2501_04684_gb300 as ie
 import workloads as W
+from gpu_util import dev, empty, host, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -61,3 +62,34 @@ def test_reading_networks_back_takes_a_bounded_scratch():
         assert _pool_high() - start <= 16 << 20         # all of them take n * 198 KB
         for a, b in zip(w, back):
             assert np.array_equal(a, b)
+
+
+def test_a_plan_that_fits_without_the_convolution_is_made_without_it():
+    p = _problem(8, 64)
+    mask = ie.precmask(ie.IE_PREC_FP32)
+    with ie.Plan(ie.problem_from(p, mask, symmetry=1)) as plan:
+        assert ie.ie_plan_far_bytes(plan.handle, ie.IE_FULL, ie.IE_PREC_FP32, 1) > 0
+        with_conv = plan.stats["device_bytes"]
+        c = dev(W.coefficients(p, 1, 1020))
+        y = empty((1, p.n))
+        ie.ie_matvec(plan.handle, ie.IE_FULL, ie.IE_PREC_FP32, c, y, 1)
+        ref = host(y)
+    q = _problem(8, 64, edge=16.0)                      # box edge lambda / 16: block products only
+    with ie.Plan(ie.problem_from(q, mask, symmetry=1)) as plan:
+        assert ie.ie_plan_far_bytes(plan.handle, ie.IE_FULL, ie.IE_PREC_FP32, 1) == 0
+        without = plan.stats["device_bytes"]
+    assert with_conv - without > 256 << 20
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    keep = without + (with_conv - without) // 2
+    fill = torch.empty(free - keep, dtype=torch.uint8, device="cuda")
+    try:
+        with ie.Plan(ie.problem_from(p, mask, symmetry=1)) as plan:
+            assert ie.ie_plan_far_bytes(plan.handle, ie.IE_FULL, ie.IE_PREC_FP32, 1) == 0
+            y.zero_()
+            ie.ie_matvec(plan.handle, ie.IE_FULL, ie.IE_PREC_FP32, c, y, 1)
+            assert rel_l2(host(y), ref) <= 2e-6
+    finally:
+        del fill
+        torch.cuda.empty_cache()
