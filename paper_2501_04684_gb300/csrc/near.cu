@@ -17,10 +17,10 @@ constexpr int kNearWarps = 8;
 // owns rows l, l + 32, ... (ROWS of them, na <= 32 ROWS); the block's source coefficients sit in
 // the warp's part of shared memory.  Columns go in groups of G whose loads are all issued before
 // the group's arithmetic, so each lane keeps G x ROWS independent reads in flight.  Per block
-// the sums run in FP32 and are added to two-float per-warp totals, combined in FP64 (the highs; the
-// lows' sum in FP32).
+// the sums run in FP32 and are added to two-float per-warp totals, combined in FP64 (the highs,
+// converted by all warps: a conversion takes as long as an FP64 addition; the lows' sum in FP32).
 // Measured (shell32, 729 MB of blocks): 128 us = 5.7 TB/s (156 us with shuffled coefficients, 16
-// columns in flight and FP64 totals); 8 scatterers, 64-row boxes, four columns: 510 us for 1.25
+// columns in flight and FP64 totals); 8 scatterers, 64-row boxes, four columns: 497 us for 1.25
 // GB (935 us with a pass over the blocks per column; in pairs of columns per CTA 552 us).
 // Nblk holds the blocks; with box_cols, columns r >= box_cols[a] take Nbeyond's instead.
 static_assert(2 * ((27 + kNearWarps - 1) / kNearWarps) <= kTotalTerms, "a warp's blocks, short and beyond");
@@ -34,8 +34,8 @@ near_kernel(const int32_t *__restrict__ nb, const int64_t *__restrict__ off, int
     if (gate && *gate == 0) return;
     constexpr int G = ROWS == 1 ? 16 : (ROWS == 2 ? 8 : 4);     // columns per load group
     constexpr int X = 32 * ROWS;
-    __shared__ __align__(16) float2 xs[kNearWarps][NR][X];      // c_b of the warp's block
-    __shared__ float4 part[kNearWarps][X];                      // (hi, lo) of re and im
+    __shared__ __align__(16) float2 xs[kNearWarps][NR][X];      // c_b of the warp's block; then lows
+    __shared__ double2 part[kNearWarps][X];                     // the totals' highs (lows: in xs)
     const int groups = (nrhs + NR - 1) / NR;             // a box's columns run next to each other
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
         const int a = item / groups, r0 = (item - a * groups) * NR;
@@ -131,8 +131,10 @@ near_kernel(const int32_t *__restrict__ nb, const int64_t *__restrict__ off, int
         for (int r = 0; r < NR; ++r) {
             __syncthreads();            // the sums before have been read
 #pragma unroll
-            for (int k = 0; k < ROWS; ++k)
-                part[warp][lane + 32 * k] = make_float4(hi[k][r].x, lo[k][r].x, hi[k][r].y, lo[k][r].y);
+            for (int k = 0; k < ROWS; ++k) {
+                part[warp][lane + 32 * k] = make_double2(hi[k][r].x, hi[k][r].y);
+                xs[warp][0][lane + 32 * k] = make_float2(low_of(hi[k][r].x, lo[k][r].x), low_of(hi[k][r].y, lo[k][r].y));
+            }
             __syncthreads();
             if (r0 + r < nrhs)
                 for (int i = threadIdx.x; i < na; i += blockDim.x) {
@@ -140,9 +142,8 @@ near_kernel(const int32_t *__restrict__ nb, const int64_t *__restrict__ off, int
                     float lr = 0.f, li = 0.f;           // the lows' own sums: 2^-24 of the totals
 #pragma unroll
                     for (int w = 0; w < kNearWarps; ++w) {
-                        const float4 q = part[w][i];
-                        sr += q.x, lr += low_of(q.x, q.y);
-                        si += q.z, li += low_of(q.z, q.w);
+                        sr += part[w][i].x, lr += xs[w][0][i].x;
+                        si += part[w][i].y, li += xs[w][0][i].y;
                     }
                     sr = kTotalTerms * (sr + lr);
                     si = kTotalTerms * (si + li);
@@ -152,6 +153,7 @@ near_kernel(const int32_t *__restrict__ nb, const int64_t *__restrict__ off, int
                     y[at] = make_float2((float)(sr + alpha * x.x), (float)(si + alpha * x.y));
                 }
         }
+        if (item + (int)gridDim.x < items) __syncthreads();         // xs has been read
     }
 }
 
