@@ -469,9 +469,9 @@ ie_status work_list(ie_plan p, bool tc, int nrhs, WorkList **out, int max_cols, 
         int64_t q = s;
         while (q < e) {
             const int nr = nr_of(q);
-            const int per = cols / nr;
-            int np = 0;
-            while (q + np < e && np < per && nr_of(q + np) == nr) ++np;
+            int np = (int)std::min<int64_t>(cols / nr, e - q);
+            for (int k = 1; k < np && !p->gnrhs.empty(); ++k)
+                if (nr_of(q + k) != nr) np = k;
             emit(pack ? p->h_pgroup[q] : d, q, np, nr);
             q += np;
         }
@@ -622,7 +622,7 @@ static ie_status chosen_translate(ie_plan p, int prec, const float2 *X, int nrhs
         IE_TRY(conv);
         const int profile = p->profile;
         p->profile = 0;                             // the bracket is this one
-        const ie_status blocks = block_translate(p, prec, X, nrhs, st, p->d_form + 1, 2 * p->tc_sms);
+        const ie_status blocks = block_translate(p, prec, X, nrhs, st, p->d_form + 1, 4 * p->tc_sms);
         p->profile = profile;
         return blocks;
     }));

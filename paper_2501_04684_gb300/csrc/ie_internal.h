@@ -378,8 +378,8 @@ ie_status adj_list(ie_plan p, bool tc, int nrhs, WorkList **out);
 ie_status launch_aggregate(const ie_plan p, const float2 *c, float2 *X, int nrhs, cudaStream_t st,
                            const int *gate = nullptr);
 // symmetry = 1: the 48 signed-permuted FP32 copies of X into p->d_Xsym
-// most_ctas here and below: at most so many CTAs (per column) that loop, for launches that are
-// mostly gated off
+// most_ctas here and below: about so many CTAs at most, which loop, for launches that are mostly
+// gated off
 ie_status launch_permute_sym(const ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate = nullptr,
                              int most_ctas = INT32_MAX);
 // plain: without the symmetric store's permuted copies

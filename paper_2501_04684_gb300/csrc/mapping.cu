@@ -412,7 +412,8 @@ ie_status launch_aggregate(const ie_plan p, const float2 *c, float2 *X, int nrhs
 ie_status launch_split_tc(const ie_plan p, const float2 *X, int nrhs, bool fp16, cudaStream_t st, const int *gate,
                           bool plain, int most_ctas) {
     const bool sym = p->sym && !plain;
-    const dim3 grid(std::min(p->nbox, most_ctas), nrhs, sym ? kSym / kSplitCopies : 1);
+    const int copies = sym ? kSym / kSplitCopies : 1;
+    const dim3 grid(std::min(p->nbox, std::max(1, most_ctas / (nrhs * copies))), nrhs, copies);
     const uint16_t *map = sym ? p->d_symmap : nullptr;
     if (fp16)
         split_kernel<true><<<grid, kNU, 0, st>>>(X, p->nbox, nrhs, p->d_Xtc, p->d_Xexp, p->d_Xinf, map, gate);
@@ -437,8 +438,10 @@ __global__ void permute_sym_kernel(const float2 *__restrict__ X, int nbox, int n
     }
 }
 
-ie_status launch_permute_sym(const ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate, int most_ctas) {
-    permute_sym_kernel<<<dim3(std::min(p->nbox, most_ctas), nrhs, kSym), kNU, 0, st>>>(X, p->nbox, nrhs, p->d_symmap, p->d_Xsym, gate);
+ie_status launch_permute_sym(const ie_plan p, const float2 *X, int nrhs, cudaStream_t st, const int *gate,
+                             int most_ctas) {
+    const dim3 grid(std::min(p->nbox, std::max(1, most_ctas / (nrhs * kSym))), nrhs, kSym);
+    permute_sym_kernel<<<grid, kNU, 0, st>>>(X, p->nbox, nrhs, p->d_symmap, p->d_Xsym, gate);
     IE_CK_LAUNCH();
     return IE_OK;
 }
@@ -483,7 +486,7 @@ ie_status launch_zero_slabs(float2 *base, int nslab, size_t stride, size_t count
     }
     const int64_t n4 = (int64_t)(count * sizeof(float2) / 16);
     int64_t gx = (n4 + 255) / 256;
-    gx = std::min<int64_t>(gx, std::min(1024, most_ctas));
+    gx = std::min<int64_t>(gx, std::min(1024, std::max(1, most_ctas / nslab)));
     zero_slabs_kernel<<<dim3((unsigned)gx, (unsigned)nslab), 256, 0, st>>>(reinterpret_cast<float4 *>(base), n4,
                                                                           (int64_t)(stride * sizeof(float2) / 16),
                                                                           gate);
