@@ -71,9 +71,11 @@ typedef enum {
  *  BF16X3  tcgen05 tensor cores, each FP32 operand split into bf16 hi + lo and the
  *          three products hi*hi + hi*lo + lo*hi accumulated in FP32.
  *  FP16X3  as BF16X3 with fp16 halves.
- *  BF16X1  tcgen05, one bf16 product (hi*hi) — the cheapest, least accurate form.
+ *  BF16X1  tcgen05, one bf16 product (hi*hi) — the cheapest, least accurate block product.
  *  FP16X1  tcgen05, one fp16 product (hi*hi) from the FP16X3 store: three more bits
  *          than BF16X1; with FP16X3 it makes a mixed pair that shares one store.
+ *          BF16X1 and FP16X1 always run per far pair; where a convolution serves the other
+ *          block precisions (below), those are both faster and more accurate.
  *  CVFCNN  the translation surrogate of §3: per stored block a complex network
  *          192 -> H -> 192 (input scaled by its l-infinity norm, one hidden layer
  *          with the Cartesian ReLU max(Re z, 0) + j max(Im z, 0), linear output,
@@ -171,8 +173,8 @@ typedef struct {
     int64_t n_far_pairs;       /* ordered (basis box, test box) far pairs             */
     int64_t n_far_disp;        /* distinct far displacements (= coupling blocks)      */
     int64_t n_near_pairs;      /* stored near blocks (self blocks included)           */
-    int64_t n_work_simt;       /* work items of the FP32 translation                  */
-    int64_t n_work_tc;         /* work items of the tensor-core translation           */
+    int64_t n_work_simt;       /* work items of the FP32 block products (0 before one)*/
+    int64_t n_work_tc;         /* ... of the tensor-core block products               */
     size_t device_bytes;       /* device memory the plan holds                        */
     double plan_seconds;       /* host wall time of ie_plan_create                    */
     double translate_ms;       /* with profiling on: summed device time of the
@@ -251,22 +253,24 @@ ie_status ie_plan_footprint_shared(const ie_problem *prob, ie_store store, size_
 
 ie_status ie_plan_stats_get(ie_plan plan, ie_plan_stats *out);
 
-/* Bytes per product that the far part of `which` (IE_FAR or IE_FULL) moves through device
- * memory when it is evaluated as a lattice convolution (its five passes, their multiplier
- * once), or 0 when this plan uses the block products for it.  Host only.
+/* Bytes per product that the convolution of `which` (IE_FAR or IE_FULL) reads and writes (its
+ * five passes' workspace, in L2 where it fits there, and their multiplier once), or 0 when this
+ * plan uses the block products for it.  An IE_FAR call whose inputs are uneven takes the block
+ * products in either case (see ie_prec).  Host only.
  * Errors: IE_ERR_INVALID, IE_ERR_UNSUPPORTED. */
 ie_status ie_plan_far_bytes(ie_plan plan, int which, int prec, int nrhs, int64_t *bytes);
 
-/* Profiling of the translation (the block-product kernel, or the convolution's passes): with enable = 1 (counters reset), every
- * translation launched outside stream capture is bracketed by CUDA events on its
- * stream and its duration added to translate_ms (the call then waits for it). */
+/* Profiling of the translation (the block-product kernel; or the convolution's passes, for far
+ * products with the choice of the form and the adjacent pairs' product): with enable = 1
+ * (counters reset), every translation launched outside stream capture is bracketed by CUDA
+ * events on its stream and its duration added to translate_ms (the call then waits for it). */
 ie_status ie_plan_profile(ie_plan plan, int enable);
 
 /* Autotuner of the tensor-core translation (no counterpart in the paper): for calls with
  * this nrhs, times the translation of precision `prec` with tile widths of 96, 80, 64
  * and 48 columns and two work-item orders (largest first; displacement order, which runs
  * the tiles of one group on neighbouring CTAs together) and keeps the fastest for the
- * plan.  Synchronises `stream`; overwrites the plan's scratch.  info (may be NULL): the
+ * plan's block products (a convolution does not use it).  Synchronises `stream`; overwrites the plan's scratch.  info (may be NULL): the
  * chosen tile width and order, its time per launch and that of the default (96, 1).
  * Errors: IE_ERR_INVALID, IE_ERR_UNSUPPORTED (FP32 or a precision not in the plan). */
 typedef struct {
@@ -324,8 +328,10 @@ ie_status ie_disaggregate(ie_plan plan, const void *Y, void *r, int nrhs, void *
  * counterpart; it serves callers that cannot allocate device memory at call time,
  * e.g. code whose device memory belongs to another allocator's pool, or a latency-
  * critical loop where cudaMalloc / cudaFree could block or synchronise the device).
- * Same arithmetic and result as ie_translate; it calls no allocator and copies nothing from host memory (the
- * displacement-group offsets it reads were put on the device with the plan).  Its
+ * It always multiplies the FP32 blocks per far pair, so where ie_translate is a convolution
+ * (see ie_prec) its result agrees to FP32 rounding and takes tens of times longer; it calls no
+ * allocator and copies nothing from host memory (the displacement-group offsets it reads were
+ * put on the device with the plan).  Its
  * scratch is a fixed 32 MiB device area inside libie (held by every GPU that loads the
  * library until exit) that must hold 8 x nrhs x n_boxes x 192 complex64 partial sums;
  * larger requests return IE_ERR_INVALID with the sizes in ie_last_error().  The first call on a device looks the area up and sets the kernel

@@ -328,7 +328,7 @@ def ie_plan_stats_get(plan: int) -> dict:
 
 
 def ie_plan_far_bytes(plan: int, which: int, prec: int, nrhs: int) -> int:
-    """Bytes per product of the convolution that evaluates the far part, 0 with block products."""
+    """Bytes the convolution of a product reads and writes (its workspace), 0 with block products."""
     b = ctypes.c_int64()
     _check(lib().ie_plan_far_bytes(plan, which, prec, nrhs, ctypes.byref(b)), "ie_plan_far_bytes")
     return b.value

@@ -608,8 +608,11 @@ ie_status prepare_conv() {
 
 // ---------------------------------------------------------------- plan
 // Bounds of the rule.  kConvKa: the transforms' rounding is relative to the whole field, so
-// the real and imaginary parts of D must be of one size for both to keep FP32 accuracy; they
-// are at a = lambda / 8 (k a = 0.785), not at lambda / 256, where the radiative part is 1e-4.
+// the real and imaginary parts of D must be of one size for both to keep FP32 accuracy.  At
+// lambda / 8 (k a = 0.785) they are (radiative part of a far product of 6^3 boxes, real moments:
+// 2.7e-7, lambda / 4 2.3e-7); at lambda / 256 the radiative part is 1e-4 of the field and a complex
+// transform would leave 1e-3 of it.  Nothing between the two is measured: the line lies just
+// below lambda / 8.
 constexpr double kConvKa = 0.75;
 // Device times (ns) of a padded lattice point here, and of a far pair and a stored block (an
 // item's chain, however few its pairs) in the block products, 16-bit split and FP32.  They
@@ -910,7 +913,7 @@ ie_status launch_choose_form(ie_plan p, const float2 *X, int nrhs, cudaStream_t 
     return IE_OK;
 }
 
-// Bytes the five passes read and write (K^ and the boxes' vectors once each).
+// Bytes the five passes read and write, in L2 or device memory (K^ and the boxes' vectors once each).
 int64_t conv_traffic(const ie_plan_s *p, int nrhs) {
     int64_t b = 2 * (int64_t)nrhs * p->nbox * kNU * sizeof(float2);
     for (const auto &c : p->conv) {

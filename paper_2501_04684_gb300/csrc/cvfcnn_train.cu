@@ -21,7 +21,7 @@
 //   A              two chunks of the matrix a product reads from global memory (cp.async)
 // The six products of a minibatch run on register tiles: 6 x 4 outputs per thread for the
 // 192-row ones (target, output layer), 4 x 2 for the 64-row ones (hidden layer, hidden
-// gradient), 7 x 6 for the two weight gradients.  FP32 rate bound, one CTA (two warps per
+// gradient), 4 x 6 for the two weight gradients (a thread's rows in two halves).  FP32 rate bound, one CTA (two warps per
 // scheduler) per SM: 192 x 192 + 5 x 192 H complex multiply-adds per sample, 0.17 ms per step
 // of 128 samples at the peak rate for H = 50; 0.43 ms measured (1.0 ms with operands
 // read per multiply-add from global memory and one gradient entry per thread at a time).
