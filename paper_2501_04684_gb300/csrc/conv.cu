@@ -622,8 +622,8 @@ constexpr double kConvKa = 0.75;
 constexpr double kPointNs = 0.03, kPairNs16 = 0.7, kBlockNs16 = 49, kPairNs32 = 6.0, kBlockNs32 = 270;
 // A far product alone also takes the adjacent pairs off (a second kernel's chain) and looks at its
 // inputs: below this many far pairs the block product is the shorter chain.  Blocks against
-// convolution, symmetric store: FP32 5,650 pairs 87 against 120 us, 13,428 pairs 143 against 103;
-// FP16X3 13,428 pairs 45 against 65 (three columns 78 against 70), 42,560 pairs 70 against 66
+// convolution, symmetric store: FP32 5,650 pairs 87 against 105 us without the look, 13,428
+// pairs 143 against 103 with it; FP16X3 13,428 pairs 45 against 65 (three columns 78 against 70), 42,560 pairs 70 against 66
 // (150 against 70).  One line for all: a single 16-bit column would draw it at 40,000, several at 10,000.
 constexpr int64_t kFarPairs = 8192;
 constexpr size_t kConvWorkspace = (size_t)256 << 20;    // bytes of A and B beyond one column
